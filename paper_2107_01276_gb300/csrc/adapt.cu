@@ -357,6 +357,19 @@ struct ShiftIn {
     }
 };
 
+// The quintic at r^2 (without sigma); the FP64 form of it and of the shift
+// terms below keeps off the divides and square roots (kernels.cuh).
+template <typename R>
+__device__ __forceinline__ R kernel_w(R r2, R hinv) {
+    if constexpr (sizeof(R) == 8) {
+        R w, s;
+        qs_ws(nonzero(r2) ? r2 * frsqrt(r2) * hinv : R(0), w, s);
+        return w;
+    } else {
+        return qs_w<R>(sqrt(r2) * hinv);
+    }
+}
+
 // Summation density of every particle (Eq. sd-gather, walls included) and,
 // for the h update, the mean fluid-neighbour mass.
 template <typename R, int T>
@@ -382,7 +395,7 @@ __global__ void __launch_bounds__(128) k_density_mbar(ShiftArgs a, int want_h) {
         // the entry adds nothing (lists with a skin hold many such
         // entries); the h update's mean mass still counts it
         if (!want_h && !(r2 < R(9) * hi * hi)) continue;
-        rho += in.m[j] * qs_w<R>(sqrt(r2) * hinv);   // zero beyond 3 h_i
+        rho += in.m[j] * kernel_w<R>(r2, hinv);   // zero beyond 3 h_i
         if (check) {
             float fx, fy, fr2;
             if (!pred_mixed(a.d, a.an, pki, __ldg(&a.pk[j]), xi, yi, hid,
@@ -395,7 +408,7 @@ __global__ void __launch_bounds__(128) k_density_mbar(ShiftArgs a, int want_h) {
     if (a.w.n > 0) {
         for_each_wall<T>(a.w, i, a.d, a.an, a.pk[i], a.f[S_X][i], a.f[S_Y][i], a.f[S_H][i], tm.lane, tm.mask,
                       [&](int k, double, double, double r2) {
-            rho += (R)a.w.m[k] * qs_w<R>(sqrt((R)r2) * hinv);
+            rho += (R)a.w.m[k] * kernel_w<R>((R)r2, hinv);
         });
     }
     rho = team_sum<T>(tm.mask, rho);
@@ -425,7 +438,20 @@ __global__ void __launch_bounds__(128) k_shift_compute(ShiftArgs a) {
     const R ui = in.u[i], vi = in.v[i], pi = in.p[i];
     const R rho0 = (R)a.rho0;
     R ax = 0, ay = 0, gux = 0, guy = 0, gvx = 0, gvy = 0, gpx = 0, gpy = 0;
-    auto shift = [&](R mj, R hj, R dx, R dy, R r) {
+    auto shift = [&](R mj, R hj, R dx, R dy, R r, R rinv) {
+        if constexpr (sizeof(R) == 8) {
+            // times -40 sigma / rho0 at the end
+            const R hsinv = frcp(hi + hj);
+            R w, s;
+            qs_ws((r + r) * hsinv, w, s);
+            R ratio = w * inv_wxi;
+            ratio *= ratio;
+            const R f = mj * (R(1) + R(0.24) * ratio * ratio) *
+                        (hsinv * hsinv * hsinv) * (s * rinv);
+            ax += f * dx;
+            ay += f * dy;
+            return;
+        }
         const R hb = R(0.5) * (hi + hj), hbinv = R(1) / hb;
         R ratio = qs_w<R>(r * hbinv) * inv_wxi;
         ratio *= ratio;
@@ -446,11 +472,21 @@ __global__ void __launch_bounds__(128) k_shift_compute(ShiftArgs a) {
             const R R3 = R(3) * (hi > hj ? hi : hj);
             if (!(r2 < R3 * R3)) continue;
         }
-        const R r = sqrt(r2);
-        if (!(r > R(0))) continue;
-        shift(in.m[j], hj, dx, dy, r);
-        const R g = sigma_norm<R>() * hinv * hinv * hinv * qs_dw<R>(r * hinv) / r;
-        const R Vg = (in.m[j] / rhoj[j]) * g;
+        R r, rinv, Vg;
+        if constexpr (sizeof(R) == 8) {
+            if (!nonzero(r2)) continue;
+            rinv = frsqrt(r2);
+            r = r2 * rinv;
+            // times -5 sigma / h_i^3 at the end
+            Vg = in.m[j] * frcp(rhoj[j]) * (qs_s(r * hinv) * rinv);
+        } else {
+            r = sqrt(r2);
+            rinv = R(0);
+            if (!(r > R(0))) continue;
+            const R g = sigma_norm<R>() * hinv * hinv * hinv * qs_dw<R>(r * hinv) / r;
+            Vg = (in.m[j] / rhoj[j]) * g;
+        }
+        shift(in.m[j], hj, dx, dy, r, rinv);
         const R du = in.u[j] - ui, dv = in.v[j] - vi, dp = in.p[j] - pi;
         gux += Vg * du * dx;
         guy += Vg * du * dy;
@@ -464,7 +500,7 @@ __global__ void __launch_bounds__(128) k_shift_compute(ShiftArgs a) {
                       [&](int k, double dxd, double dyd, double r2) {
             const R r = sqrt((R)r2);
             if (!(r > R(0))) return;
-            shift((R)a.w.m[k], (R)a.w.h[k], (R)dxd, (R)dyd, r);
+            shift((R)a.w.m[k], (R)a.w.h[k], (R)dxd, (R)dyd, r, R(1) / r);
         });
     }
     ax = team_sum<T>(tm.mask, ax);
@@ -476,7 +512,17 @@ __global__ void __launch_bounds__(128) k_shift_compute(ShiftArgs a) {
     gpx = team_sum<T>(tm.mask, gpx);
     gpy = team_sum<T>(tm.mask, gpy);
     if (tm.lane != 0) return;
-    const R c = R(-0.5) * hi * hi;
+    R c = R(-0.5) * hi * hi;
+    if constexpr (sizeof(R) == 8) {
+        c *= R(-40) * sigma_norm<R>() / rho0;
+        const R k = R(-5) * sigma_norm<R>() * hinv * hinv * hinv;
+        gux *= k;
+        guy *= k;
+        gvx *= k;
+        gvy *= k;
+        gpx *= k;
+        gpy *= k;
+    }
     R sx = c * ax, sy = c * ay;
     const R mag = sqrt(sx * sx + sy * sy), lim = R(0.25) * hi;
     if (mag > lim) {

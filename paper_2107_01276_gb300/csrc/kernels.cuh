@@ -33,12 +33,52 @@ __device__ __forceinline__ R qs_dw(R q) {
     return R(-5) * (a2 * a2) + R(30) * (b2 * b2) - R(75) * (c2 * c2);
 }
 
-// a / b and 1/sqrt(x): IEEE in double; the fast FP32 forms (at most 2 ulp)
-// in float, well inside the mixed path's tolerance.
-__device__ __forceinline__ double fdiv(double a, double b) { return a / b; }
+// a / b and 1/sqrt(x).  Float: the fast FP32 forms (at most 2 ulp), well
+// inside the mixed path's tolerance.  Double: the hardware's 20-bit
+// estimate refined by one third-order Householder step, with e = 1 - b y
+// (reciprocal) or 1 - x y^2 (reciprocal square root) of at most 2^-19: the
+// remainder e^3 lies below half an ulp, so the result is within 1.5 ulp for
+// normal operands and results.  GB300 issues one FP64 instruction per SM
+// sub-partition every 64 cycles, and the pair sums are bound by that pipe:
+// the correctly rounded divide and square root cost it tens of
+// instructions a pair, these three and five.
+__device__ __forceinline__ double frcp(double b) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
+    const double e = __fma_rn(-b, y, 1.0);
+    return __fma_rn(y, __fma_rn(e, e, e), y);
+}
+__device__ __forceinline__ double frsqrt(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = __fma_rn(-__dmul_rn(x, y), y, 1.0);
+    return __fma_rn(__dmul_rn(y, e), __fma_rn(0.375, e, 0.5), y);
+}
+__device__ __forceinline__ double fdiv(double a, double b) { return a * frcp(b); }
 __device__ __forceinline__ float fdiv(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double frsqrt(double x) { return 1.0 / sqrt(x); }
 __device__ __forceinline__ float frsqrt(float x) { return rsqrtf(x); }
+
+// FP64 pair sums: max(t, 0) for t <= 3 on the integer pipe (a NaN or a
+// negative t gives zero, like clip0), and the quintic with its bases shared
+// between value and derivative: w = a^5 - 6 b^5 + 15 c^5, s = a^4 - 6 b^4 +
+// 15 c^4, dw/dq = -5 s.
+__device__ __forceinline__ double clip3(double t) {
+    return (unsigned)__double2hiint(t) > 0x40080000u ? 0.0 : t;
+}
+__device__ __forceinline__ double qs_s(double q) {
+    const double a = clip3(3.0 - q), b = clip3(2.0 - q), c = clip3(1.0 - q);
+    const double a2 = a * a, b2 = b * b, c2 = c * c;
+    return __fma_rn(a2, a2, __fma_rn(-6.0 * b2, b2, 15.0 * c2 * c2));
+}
+__device__ __forceinline__ void qs_ws(double q, double &w, double &s) {
+    const double a = clip3(3.0 - q), b = clip3(2.0 - q), c = clip3(1.0 - q);
+    const double a2 = a * a, b2 = b * b, c2 = c * c;
+    const double a4 = a2 * a2, B = -6.0 * b2 * b2, C = 15.0 * c2 * c2;
+    w = __fma_rn(a4, a, __fma_rn(B, b, C * c));
+    s = a4 + (B + C);
+}
+// x != 0 for x >= 0, on the integer pipe
+__device__ __forceinline__ bool nonzero(double x) { return __double_as_longlong(x) != 0; }
 
 // Four values of one neighbour, loaded together.
 template <typename R> struct V4;

@@ -64,6 +64,28 @@ struct PassALane {
     // member j (self: j == i) at separation r_i - r_j = (dx, dy), r2 = r^2
     __device__ __forceinline__ void pair(R mj, R hj, R pj, bool self, R dx,
                                          R dy, R r2) {
+        if constexpr (sizeof(R) == 8) {
+            // r = 0 (i itself): rinv = 0 and the shift term is zero
+            const R rinv = nonzero(r2) ? frsqrt(r2) : R(0);
+            const R r = r2 * rinv;
+            R w, s;
+            qs_ws(r * hinv, w, s);
+            rho += mj * w;
+            srw += (mj * r) * s;          // times -5 in finish()
+            psum += pj;
+            cnt += 1;
+            const R hsinv = frcp(hi + hj);
+            qs_ws((r + r) * hsinv, w, s);
+            R ratio = w * inv_wxi;
+            ratio *= ratio;
+            // sigma (2 / (h_i + h_j))^3 times -5 s: the constants -40
+            // sigma are applied in finish()
+            const R f = mj * (R(1) + R(0.24) * ratio * ratio) *
+                        (hsinv * hsinv * hsinv) * (s * rinv);
+            ax += f * dx;
+            ay += f * dy;
+            return;
+        }
         const R rinv = r2 > R(0) ? frsqrt(r2) : R(0);
         const R r = r2 * rinv;
         const R q = r * hinv;
@@ -108,6 +130,11 @@ struct PassALane {
         ay = team_sum<T>(tm.mask, ay);
         cnt = team_sum<T>(tm.mask, cnt);
         if (tm.lane != 0) return;
+        if constexpr (sizeof(R) == 8) {
+            srw *= R(-5);
+            ax *= R(-40) * sigma_norm<R>();
+            ay *= R(-40) * sigma_norm<R>();
+        }
         const R sig = sigma_norm<R>() * hinv * hinv;
         rho *= sig;
         const R beta = -(sig * hinv * srw) / (rho * R(2));
@@ -196,7 +223,13 @@ struct PassBLane {
                                          R Vj, R rho_j, R Pj, R pj, R ujx,
                                          R ujy, R ugx, R ugy) {
         R gi = 0, gj = 0;
-        if (r2 > R(0)) {
+        if constexpr (sizeof(R) == 8) {
+            const R rinv = nonzero(r2) ? frsqrt(r2) : R(0);
+            const R r = r2 * rinv;
+            const R k = R(-5) * rinv;
+            gi = dsig_i * (qs_s(r * hinv) * k);
+            gj = (sigma_norm<R>() * hjinv) * (hjinv * hjinv) * (qs_s(r * hjinv) * k);
+        } else if (r2 > R(0)) {
             const R rinv = frsqrt(r2);
             const R r = r2 * rinv;
             gi = dsig_i * qs_dw<R>(r * hinv) * rinv;

@@ -102,10 +102,13 @@ __host__ __device__ inline uint32_t hash_slot(uint64_t k, uint32_t mask) {
     return (uint32_t)k & mask;
 }
 
-// Minimum-image separation component, FP64, no contraction.
+// Minimum-image separation component, FP64, no contraction.  A separation
+// whose high word is below the half period's is already the minimum image
+// (most pairs): that test runs on the integer pipe.
 __device__ __forceinline__ double min_image(const Domain &d, int a,
                                             double s) {
-    if (d.periodic[a]) {
+    if (d.periodic[a] &&
+        (__double2hiint(s) & 0x7fffffff) >= __double2hiint(d.half[a])) {
         if (s > d.half[a])
             s = __dsub_rn(s, d.L[a]);
         else if (s < -d.half[a])
