@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(128) k_shift_compute(ShiftArgs a) {
             // times -40 sigma / rho0 at the end
             const R hsinv = frcp(hi + hj);
             R w, s;
-            qs_ws((r + r) * hsinv, w, s);
+            qs_ws(__dmul_rn(r + r, hsinv), w, s);
             R ratio = w * inv_wxi;
             ratio *= ratio;
             const R f = mj * (R(1) + R(0.24) * ratio * ratio) *
@@ -476,9 +476,9 @@ __global__ void __launch_bounds__(128) k_shift_compute(ShiftArgs a) {
         if constexpr (sizeof(R) == 8) {
             if (!nonzero(r2)) continue;
             rinv = frsqrt(r2);
-            r = r2 * rinv;
+            r = __dmul_rn(r2, rinv);
             // times -5 sigma / h_i^3 at the end
-            Vg = in.m[j] * frcp(rhoj[j]) * (qs_s(r * hinv) * rinv);
+            Vg = in.m[j] * frcp(rhoj[j]) * (qs_s(__dmul_rn(r, hinv)) * rinv);
         } else {
             r = sqrt(r2);
             rinv = R(0);

@@ -67,21 +67,21 @@ struct PassALane {
         if constexpr (sizeof(R) == 8) {
             // r = 0 (i itself): rinv = 0 and the shift term is zero
             const R rinv = nonzero(r2) ? frsqrt(r2) : R(0);
-            const R r = r2 * rinv;
+            const R r = __dmul_rn(r2, rinv);
             R w, s;
-            qs_ws(r * hinv, w, s);
+            qs_ws(__dmul_rn(r, hinv), w, s);
             rho += mj * w;
-            srw += (mj * r) * s;          // times -5 in finish()
+            srw += __dmul_rn(mj, r) * s;  // times -5 in finish()
             psum += pj;
             cnt += 1;
             const R hsinv = frcp(hi + hj);
-            qs_ws((r + r) * hsinv, w, s);
-            R ratio = w * inv_wxi;
-            ratio *= ratio;
+            qs_ws(__dmul_rn(r + r, hsinv), w, s);
+            R ratio = __dmul_rn(w, inv_wxi);
+            ratio = __dmul_rn(ratio, ratio);
             // sigma (2 / (h_i + h_j))^3 times -5 s: the constants -40
             // sigma are applied in finish()
-            const R f = mj * (R(1) + R(0.24) * ratio * ratio) *
-                        (hsinv * hsinv * hsinv) * (s * rinv);
+            const R f = mj * __fma_rn(__dmul_rn(R(0.24), ratio), ratio, R(1)) *
+                        (hsinv * hsinv * hsinv) * __dmul_rn(s, rinv);
             ax += f * dx;
             ay += f * dy;
             return;
@@ -144,7 +144,7 @@ struct PassALane {
             drx = c * ax;
             dry = c * ay;
         }
-        const R mag = sqrt(drx * drx + dry * dry);
+        const R mag = sizeof(R) == 8 ? sqrt(mad2(drx, drx, dry, dry)) : sqrt(drx * drx + dry * dry);
         const R lim = R(0.25) * hi;
         if (mag > lim) {
             const R th = lim / mag;
@@ -193,7 +193,7 @@ struct PassALane {
 template <typename R>
 struct PassBLane {
     R hinv, dsig_i, rho_i, pi, ui, vi, pavg_i, Pi, eta;
-    bool dden_on;
+    bool dden_on, visc_on;
     R div, diff, fax, fay, vx, vy;
 
     // false: beta_i = 0 (no neighbour at r > 0), zero rates (reading R1)
@@ -204,7 +204,7 @@ struct PassBLane {
         if (beta_i == R(0)) return false;
         const typename V4<R>::T Bi = a.nbB[i];
         hinv = Bi.w;
-        dsig_i = sigma_norm<R>() * hinv * hinv * hinv;
+        dsig_i = (sizeof(R) == 8 ? R(1) : sigma_norm<R>()) * hinv * hinv * hinv;
         rho_i = a.rho[i];
         pi = Bi.x;
         ui = Bi.y;
@@ -214,6 +214,7 @@ struct PassBLane {
         const R hi = R(1) / hinv;
         eta = R(0.001) * hi * hi;
         dden_on = a.diff_denominator != 0;
+        visc_on = a.nu != 0.0;
         return true;
     }
 
@@ -225,10 +226,11 @@ struct PassBLane {
         R gi = 0, gj = 0;
         if constexpr (sizeof(R) == 8) {
             const R rinv = nonzero(r2) ? frsqrt(r2) : R(0);
-            const R r = r2 * rinv;
-            const R k = R(-5) * rinv;
-            gi = dsig_i * (qs_s(r * hinv) * k);
-            gj = (sigma_norm<R>() * hjinv) * (hjinv * hjinv) * (qs_s(r * hjinv) * k);
+            const R r = __dmul_rn(r2, rinv);
+            const R k = R(-5) * sigma_norm<R>() * rinv;
+            // dsig_i: 1 / h_i^3
+            gi = __dmul_rn(qs_s(__dmul_rn(r, hinv)) * k, dsig_i);
+            gj = __dmul_rn(qs_s(__dmul_rn(r, hjinv)) * k, hjinv * hjinv * hjinv);
         } else if (r2 > R(0)) {
             const R rinv = frsqrt(r2);
             const R r = r2 * rinv;
@@ -241,12 +243,17 @@ struct PassBLane {
         const R nu_ij = fdiv(R(1), hinv + hjinv);
         const R inv_reta = fdiv(R(1), r2 + eta);
         const R uij = ui - ujx, vij = vi - ujy;
-        div += Vj * gi * (uij * dx + vij * dy);
+        if constexpr (sizeof(R) == 8)
+            div += Vj * gi * mad2(uij, dx, vij, dy);
+        else
+            div += Vj * gi * (uij * dx + vij * dy);
         diff += Vj * nu_ij * (pi - pj) * rdg * (dden_on ? inv_reta : R(1));
-        const R mfp = mj * (Pi * gi + Pj * gj);
+        const R mfp = sizeof(R) == 8 ? mj * mad2(Pi, gi, Pj, gj) : mj * (Pi * gi + Pj * gj);
         fax -= mfp * dx;
         fay -= mfp * dy;
         // m_j 4 nu/(rho_i + rho_j) r.gW_ij/(r^2 + eta) / (4 nu)
+        // (an inviscid flow's sum is multiplied by zero in finish())
+        if (sizeof(R) == 8 && !visc_on) return;
         const R visc = fdiv(mj * rdg * inv_reta, rho_i + rho_j);
         vx += visc * (ui - ugx);
         vy += visc * (vi - ugy);
@@ -300,7 +307,8 @@ struct PassBLane {
         const R rf = a.rho_factor ? rho_i : R(1);
         // (u~ - u) = dr / dt by the reciprocal the time-step kernel stores
         const R idt = (R)a.dt[1];
-        const R tvf = -(a.drx[i] * idt * fax + a.dry[i] * idt * fay);
+        const R tvf = sizeof(R) == 8 ? -mad2(a.drx[i] * idt, fax, a.dry[i] * idt, fay)
+                                     : -(a.drx[i] * idt * fax + a.dry[i] * idt * fay);
         const R half_ac = R(0.5) * (R)a.alpha_e * (R)a.cs;
         const R four_nu = R(4) * (R)a.nu;
         const R dpdt = ((R)a.rho0 * (R)a.cs * (R)a.cs / beta_i) * div +
