@@ -357,22 +357,10 @@ struct ShiftIn {
     }
 };
 
-// The quintic at r^2 (without sigma); the FP64 form of it and of the shift
-// terms below keeps off the divides and square roots (kernels.cuh).
-template <typename R>
-__device__ __forceinline__ R kernel_w(R r2, R hinv) {
-    if constexpr (sizeof(R) == 8) {
-        R w, s;
-        qs_ws(nonzero(r2) ? r2 * frsqrt(r2) * hinv : R(0), w, s);
-        return w;
-    } else {
-        return qs_w<R>(sqrt(r2) * hinv);
-    }
-}
-
 // Summation density of every particle (Eq. sd-gather, walls included) and,
-// for the h update, the mean fluid-neighbour mass.
-template <typename R, int T>
+// for the h update, the mean fluid-neighbour mass.  LEAN: a set without
+// walls, whose FP64 sums keep off the divides and square roots (kernels.cuh).
+template <typename R, int T, bool LEAN>
 __global__ void __launch_bounds__(128) k_density_mbar(ShiftArgs a, int want_h) {
     const Team<T> tm;
     const int i = Team<T>::particle();
@@ -395,7 +383,13 @@ __global__ void __launch_bounds__(128) k_density_mbar(ShiftArgs a, int want_h) {
         // the entry adds nothing (lists with a skin hold many such
         // entries); the h update's mean mass still counts it
         if (!want_h && !(r2 < R(9) * hi * hi)) continue;
-        rho += in.m[j] * kernel_w<R>(r2, hinv);   // zero beyond 3 h_i
+        if constexpr (lean64<R, LEAN>) {
+            R w, s;
+            qs_ws(nonzero(r2) ? __dmul_rn(__dmul_rn(r2, frsqrt_lean(r2)), hinv) : R(0), w, s);
+            rho += in.m[j] * w;
+        } else {
+            rho += in.m[j] * qs_w<R>(sqrt(r2) * hinv);   // zero beyond 3 h_i
+        }
         if (check) {
             float fx, fy, fr2;
             if (!pred_mixed(a.d, a.an, pki, __ldg(&a.pk[j]), xi, yi, hid,
@@ -408,7 +402,7 @@ __global__ void __launch_bounds__(128) k_density_mbar(ShiftArgs a, int want_h) {
     if (a.w.n > 0) {
         for_each_wall<T>(a.w, i, a.d, a.an, a.pk[i], a.f[S_X][i], a.f[S_Y][i], a.f[S_H][i], tm.lane, tm.mask,
                       [&](int k, double, double, double r2) {
-            rho += (R)a.w.m[k] * kernel_w<R>((R)r2, hinv);
+            rho += (R)a.w.m[k] * qs_w<R>(sqrt((R)r2) * hinv);
         });
     }
     rho = team_sum<T>(tm.mask, rho);
@@ -424,7 +418,7 @@ __global__ void __launch_bounds__(128) k_density_mbar(ShiftArgs a, int want_h) {
 // Limited shift (Eqs. shift-deltar, shift-limit; walls included) and the
 // Taylor increments grad phi_i . dr_i with grad phi_i = sum_{j != i} V_j
 // (phi_j - phi_i) grad_i W(r_ij, h_i) over fluid neighbours.
-template <typename R, int T>
+template <typename R, int T, bool LEAN>
 __global__ void __launch_bounds__(128) k_shift_compute(ShiftArgs a) {
     const Team<T> tm;
     const int i = Team<T>::particle();
@@ -438,20 +432,7 @@ __global__ void __launch_bounds__(128) k_shift_compute(ShiftArgs a) {
     const R ui = in.u[i], vi = in.v[i], pi = in.p[i];
     const R rho0 = (R)a.rho0;
     R ax = 0, ay = 0, gux = 0, guy = 0, gvx = 0, gvy = 0, gpx = 0, gpy = 0;
-    auto shift = [&](R mj, R hj, R dx, R dy, R r, R rinv) {
-        if constexpr (sizeof(R) == 8) {
-            // times -40 sigma / rho0 at the end
-            const R hsinv = frcp(hi + hj);
-            R w, s;
-            qs_ws(__dmul_rn(r + r, hsinv), w, s);
-            R ratio = w * inv_wxi;
-            ratio *= ratio;
-            const R f = mj * (R(1) + R(0.24) * ratio * ratio) *
-                        (hsinv * hsinv * hsinv) * (s * rinv);
-            ax += f * dx;
-            ay += f * dy;
-            return;
-        }
+    auto shift = [&](R mj, R hj, R dx, R dy, R r) {
         const R hb = R(0.5) * (hi + hj), hbinv = R(1) / hb;
         R ratio = qs_w<R>(r * hbinv) * inv_wxi;
         ratio *= ratio;
@@ -472,21 +453,29 @@ __global__ void __launch_bounds__(128) k_shift_compute(ShiftArgs a) {
             const R R3 = R(3) * (hi > hj ? hi : hj);
             if (!(r2 < R3 * R3)) continue;
         }
-        R r, rinv, Vg;
-        if constexpr (sizeof(R) == 8) {
+        R Vg;
+        if constexpr (lean64<R, LEAN>) {
             if (!nonzero(r2)) continue;
-            rinv = frsqrt(r2);
-            r = __dmul_rn(r2, rinv);
+            const R rinv = frsqrt_lean(r2), r = __dmul_rn(r2, rinv);
+            // times -40 sigma / rho0 at the end
+            const R hsinv = frcp(hi + hj);
+            R w, s;
+            qs_ws(__dmul_rn(r + r, hsinv), w, s);
+            R ratio = __dmul_rn(w, inv_wxi);
+            ratio = __dmul_rn(ratio, ratio);
+            const R f = in.m[j] * __fma_rn(__dmul_rn(R(0.24), ratio), ratio, R(1)) *
+                        (hsinv * hsinv * hsinv) * __dmul_rn(s, rinv);
+            ax += f * dx;
+            ay += f * dy;
             // times -5 sigma / h_i^3 at the end
             Vg = in.m[j] * frcp(rhoj[j]) * (qs_s(__dmul_rn(r, hinv)) * rinv);
         } else {
-            r = sqrt(r2);
-            rinv = R(0);
+            const R r = sqrt(r2);
             if (!(r > R(0))) continue;
+            shift(in.m[j], hj, dx, dy, r);
             const R g = sigma_norm<R>() * hinv * hinv * hinv * qs_dw<R>(r * hinv) / r;
             Vg = (in.m[j] / rhoj[j]) * g;
         }
-        shift(in.m[j], hj, dx, dy, r, rinv);
         const R du = in.u[j] - ui, dv = in.v[j] - vi, dp = in.p[j] - pi;
         gux += Vg * du * dx;
         guy += Vg * du * dy;
@@ -500,7 +489,7 @@ __global__ void __launch_bounds__(128) k_shift_compute(ShiftArgs a) {
                       [&](int k, double dxd, double dyd, double r2) {
             const R r = sqrt((R)r2);
             if (!(r > R(0))) return;
-            shift((R)a.w.m[k], (R)a.w.h[k], (R)dxd, (R)dyd, r, R(1) / r);
+            shift((R)a.w.m[k], (R)a.w.h[k], (R)dxd, (R)dyd, r);
         });
     }
     ax = team_sum<T>(tm.mask, ax);
@@ -513,7 +502,7 @@ __global__ void __launch_bounds__(128) k_shift_compute(ShiftArgs a) {
     gpy = team_sum<T>(tm.mask, gpy);
     if (tm.lane != 0) return;
     R c = R(-0.5) * hi * hi;
-    if constexpr (sizeof(R) == 8) {
+    if constexpr (lean64<R, LEAN>) {
         c *= R(-40) * sigma_norm<R>() / rho0;
         const R k = R(-5) * sigma_norm<R>() * hinv * hinv * hinv;
         gux *= k;
@@ -618,15 +607,25 @@ void launch_compact(cudaStream_t s, int n, const uint32_t *alive,
                     const uint32_t *pos, const CompactArgs &c) {
     if (n > 0) k_compact<<<nblk(n, 256), 256, 0, s>>>(n, alive, pos, c);
 }
-template <typename R, int T>
-static void shift_round_T(cudaStream_t s, const ShiftArgs &a) {
-    k_density_mbar<R, T><<<nblk(a.n * T, 128), 128, 0, s>>>(a, 0);
-    k_shift_compute<R, T><<<nblk(a.n * T, 128), 128, 0, s>>>(a);
-    k_shift_apply<R><<<nblk(a.n, 256), 256, 0, s>>>(a);
+// f(team size, LEAN) with LEAN for FP64 sets without walls.
+template <typename R, class F>
+static void with_team_lean(const ShiftArgs &a, F &&f) {
+    with_team(a.n, [&](auto t) {
+        if (sizeof(R) == 8 && a.w.n <= 0)
+            f(t, std::integral_constant<bool, sizeof(R) == 8>());
+        else
+            f(t, std::false_type());
+    });
 }
 template <typename R>
 static void shift_round_R(cudaStream_t s, const ShiftArgs &a) {
-    with_team(a.n, [&](auto t) { shift_round_T<R, decltype(t)::value>(s, a); });
+    with_team_lean<R>(a, [&](auto t, auto lean) {
+        constexpr int T = decltype(t)::value;
+        constexpr bool L = decltype(lean)::value;
+        k_density_mbar<R, T, L><<<nblk(a.n * T, 128), 128, 0, s>>>(a, 0);
+        k_shift_compute<R, T, L><<<nblk(a.n * T, 128), 128, 0, s>>>(a);
+    });
+    k_shift_apply<R><<<nblk(a.n, 256), 256, 0, s>>>(a);
 }
 void launch_shift_round(cudaStream_t s, const ShiftArgs &a, bool mixed) {
     if (a.n <= 0) return;
@@ -635,14 +634,13 @@ void launch_shift_round(cudaStream_t s, const ShiftArgs &a, bool mixed) {
     else
         shift_round_R<double>(s, a);
 }
-template <typename R, int T>
-static void h_update_T(cudaStream_t s, const ShiftArgs &a) {
-    k_density_mbar<R, T><<<nblk(a.n * T, 128), 128, 0, s>>>(a, 1);
-    k_h_apply<R><<<nblk(a.n, 256), 256, 0, s>>>(a);
-}
 template <typename R>
 static void h_update_R(cudaStream_t s, const ShiftArgs &a) {
-    with_team(a.n, [&](auto t) { h_update_T<R, decltype(t)::value>(s, a); });
+    with_team_lean<R>(a, [&](auto t, auto lean) {
+        constexpr int T = decltype(t)::value;
+        k_density_mbar<R, T, decltype(lean)::value><<<nblk(a.n * T, 128), 128, 0, s>>>(a, 1);
+    });
+    k_h_apply<R><<<nblk(a.n, 256), 256, 0, s>>>(a);
 }
 void launch_h_update(cudaStream_t s, const ShiftArgs &a, bool mixed) {
     if (a.n <= 0) return;

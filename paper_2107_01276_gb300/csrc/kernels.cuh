@@ -38,36 +38,47 @@ __device__ __forceinline__ R qs_dw(R q) {
 __device__ __forceinline__ double mad2(double a, double b, double c, double d) {
     return __fma_rn(a, b, __dmul_rn(c, d));
 }
-__device__ __forceinline__ float mad2(float a, float b, float c, float d) {
-    return __fmaf_rn(a, b, __fmul_rn(c, d));
-}
 
-// a / b and 1/sqrt(x).  Float: the fast FP32 forms (at most 2 ulp), well
-// inside the mixed path's tolerance.  Double: the hardware's 20-bit
-// estimate refined by one third-order Householder step, with e = 1 - b y
-// (reciprocal) or 1 - x y^2 (reciprocal square root) of at most 2^-19: the
-// remainder e^3 lies below half an ulp, so the result is within 1.5 ulp for
-// normal operands and results.  GB300 issues one FP64 instruction per SM
-// sub-partition every 64 cycles, and the pair sums are bound by that pipe:
-// the correctly rounded divide and square root cost it tens of
-// instructions a pair, these three and five.
+// a / b and 1/sqrt(x): IEEE in double; the fast FP32 forms (at most 2 ulp)
+// in float, well inside the mixed path's tolerance.
+__device__ __forceinline__ double fdiv(double a, double b) { return a / b; }
+__device__ __forceinline__ float fdiv(float a, float b) { return __fdividef(a, b); }
+__device__ __forceinline__ double frsqrt(double x) { return 1.0 / sqrt(x); }
+__device__ __forceinline__ float frsqrt(float x) { return rsqrtf(x); }
+
+// The FP64 pair sums of sets without walls (LEAN below) take their
+// reciprocals from the hardware's 20-bit estimate and one third-order
+// Householder step, with e = 1 - b y (reciprocal) or 1 - x y^2 (reciprocal
+// square root) of at most 2^-19: the remainder e^3 lies below half an ulp,
+// so the result is within 1.5 ulp for normal operands and results.  GB300
+// issues one FP64 instruction per SM sub-partition every 64 cycles, and the
+// pair sums are bound by that pipe: the correctly rounded divide and square
+// root cost it tens of instructions a pair, these three and five.
+//
+// Sets with walls keep the correctly rounded sequence, operation for
+// operation.  They are the adaptive flows, and adaptation amplifies a last
+// bit: a split parent's children sit on a hexagon, whose equal distances
+// the merge search orders by their rounding, so after one bit the flow
+// splits and merges other particles.  Their sums are a small part of an
+// adaptive step (pass A and B 7 % of one of the 1:250 cylinder, 91k
+// particles), and their runs keep their particle history.
+template <typename R, bool LEAN>
+constexpr bool lean64 = LEAN && sizeof(R) == 8;
+
 __device__ __forceinline__ double frcp(double b) {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
     const double e = __fma_rn(-b, y, 1.0);
     return __fma_rn(y, __fma_rn(e, e, e), y);
 }
-__device__ __forceinline__ double frsqrt(double x) {
+__device__ __forceinline__ double frsqrt_lean(double x) {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     const double e = __fma_rn(-__dmul_rn(x, y), y, 1.0);
     return __fma_rn(__dmul_rn(y, e), __fma_rn(0.375, e, 0.5), y);
 }
-__device__ __forceinline__ double fdiv(double a, double b) { return a * frcp(b); }
-__device__ __forceinline__ float fdiv(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ float frsqrt(float x) { return rsqrtf(x); }
 
-// FP64 pair sums: the quintic as one polynomial per unit piece, in t = 3 -
+// LEAN FP64 pair sums: the quintic as one polynomial per unit piece, in t = 3 -
 // q, 2 - q or 1 - q (0 <= t <= 1, so Horner's rule is well conditioned):
 //   q in [2, 3): t^5
 //   q in [1, 2): 1 + 5t + 10t^2 + 10t^3 + 5t^4 - 5t^5

@@ -47,8 +47,9 @@ __device__ __forceinline__ bool skin_member(const Domain &d, const Anchor &an,
 // limited to 0.25 h_i (Eq. shift-limit).  finish() also writes the two
 // per-particle records pass B gathers: {m, V = m/rho, rho, 1/(rho^2 beta)}
 // and {p, u, v, 1/h}.
-template <typename R>
+template <typename R, bool LEAN>
 struct PassALane {
+    static constexpr bool L64 = lean64<R, LEAN>;
     R hi, hinv, inv_wxi;
     R rho, srw, psum, ax, ay;
     int cnt;
@@ -64,9 +65,9 @@ struct PassALane {
     // member j (self: j == i) at separation r_i - r_j = (dx, dy), r2 = r^2
     __device__ __forceinline__ void pair(R mj, R hj, R pj, bool self, R dx,
                                          R dy, R r2) {
-        if constexpr (sizeof(R) == 8) {
+        if constexpr (L64) {
             // r = 0 (i itself): rinv = 0 and the shift term is zero
-            const R rinv = nonzero(r2) ? frsqrt(r2) : R(0);
+            const R rinv = nonzero(r2) ? frsqrt_lean(r2) : R(0);
             const R r = __dmul_rn(r2, rinv);
             R w, s;
             qs_ws(__dmul_rn(r, hinv), w, s);
@@ -130,7 +131,7 @@ struct PassALane {
         ay = team_sum<T>(tm.mask, ay);
         cnt = team_sum<T>(tm.mask, cnt);
         if (tm.lane != 0) return;
-        if constexpr (sizeof(R) == 8) {
+        if constexpr (L64) {
             srw *= R(-5);
             ax *= R(-40) * sigma_norm<R>();
             ay *= R(-40) * sigma_norm<R>();
@@ -144,7 +145,11 @@ struct PassALane {
             drx = c * ax;
             dry = c * ay;
         }
-        const R mag = sizeof(R) == 8 ? sqrt(mad2(drx, drx, dry, dry)) : sqrt(drx * drx + dry * dry);
+        R mag;
+        if constexpr (L64)
+            mag = sqrt(mad2(drx, drx, dry, dry));
+        else
+            mag = sqrt(drx * drx + dry * dry);
         const R lim = R(0.25) * hi;
         if (mag > lim) {
             const R th = lim / mag;
@@ -190,8 +195,9 @@ struct PassALane {
 // Cleary numerator alpha_e c / 2 of the diffusion sum, the 4 nu of the
 // viscous sum, and the transport sum, which is (dr_i/dt) . sum m_j (P_i
 // gW_i + P_j gW_j) = -(dr_i/dt) . (pressure force sum).
-template <typename R>
+template <typename R, bool LEAN>
 struct PassBLane {
+    static constexpr bool L64 = lean64<R, LEAN>;
     R hinv, dsig_i, rho_i, pi, ui, vi, pavg_i, Pi, eta;
     bool dden_on, visc_on;
     R div, diff, fax, fay, vx, vy;
@@ -204,7 +210,7 @@ struct PassBLane {
         if (beta_i == R(0)) return false;
         const typename V4<R>::T Bi = a.nbB[i];
         hinv = Bi.w;
-        dsig_i = (sizeof(R) == 8 ? R(1) : sigma_norm<R>()) * hinv * hinv * hinv;
+        dsig_i = L64 ? hinv * hinv * hinv : sigma_norm<R>() * hinv * hinv * hinv;
         rho_i = a.rho[i];
         pi = Bi.x;
         ui = Bi.y;
@@ -218,14 +224,21 @@ struct PassBLane {
         return true;
     }
 
+    __device__ __forceinline__ static R recip(R b) {
+        if constexpr (L64)
+            return frcp(b);
+        else
+            return fdiv(R(1), b);
+    }
+
     // one neighbour's contributions; (ujx, ujy): velocity in the divergence
     // sum, (ugx, ugy): velocity in the viscous sum
     __device__ __forceinline__ void pair(R dx, R dy, R r2, R hjinv, R mj,
                                          R Vj, R rho_j, R Pj, R pj, R ujx,
                                          R ujy, R ugx, R ugy) {
         R gi = 0, gj = 0;
-        if constexpr (sizeof(R) == 8) {
-            const R rinv = nonzero(r2) ? frsqrt(r2) : R(0);
+        if constexpr (L64) {
+            const R rinv = nonzero(r2) ? frsqrt_lean(r2) : R(0);
             const R r = __dmul_rn(r2, rinv);
             const R k = R(-5) * sigma_norm<R>() * rinv;
             // dsig_i: 1 / h_i^3
@@ -240,21 +253,30 @@ struct PassBLane {
         }
         const R rdg = R(0.5) * (gi + gj) * r2;
         // nu_ij / (alpha_e c / 2)
-        const R nu_ij = fdiv(R(1), hinv + hjinv);
-        const R inv_reta = fdiv(R(1), r2 + eta);
+        const R nu_ij = recip(hinv + hjinv);
+        const R inv_reta = recip(r2 + eta);
         const R uij = ui - ujx, vij = vi - ujy;
-        if constexpr (sizeof(R) == 8)
+        if constexpr (L64)
             div += Vj * gi * mad2(uij, dx, vij, dy);
         else
             div += Vj * gi * (uij * dx + vij * dy);
         diff += Vj * nu_ij * (pi - pj) * rdg * (dden_on ? inv_reta : R(1));
-        const R mfp = sizeof(R) == 8 ? mj * mad2(Pi, gi, Pj, gj) : mj * (Pi * gi + Pj * gj);
+        R mfp;
+        if constexpr (L64)
+            mfp = mj * mad2(Pi, gi, Pj, gj);
+        else
+            mfp = mj * (Pi * gi + Pj * gj);
         fax -= mfp * dx;
         fay -= mfp * dy;
         // m_j 4 nu/(rho_i + rho_j) r.gW_ij/(r^2 + eta) / (4 nu)
         // (an inviscid flow's sum is multiplied by zero in finish())
-        if (sizeof(R) == 8 && !visc_on) return;
-        const R visc = fdiv(mj * rdg * inv_reta, rho_i + rho_j);
+        R visc;
+        if constexpr (L64) {
+            if (!visc_on) return;
+            visc = mj * rdg * inv_reta * frcp(rho_i + rho_j);
+        } else {
+            visc = fdiv(mj * rdg * inv_reta, rho_i + rho_j);
+        }
         vx += visc * (ui - ugx);
         vy += visc * (vi - ugy);
     }
@@ -307,8 +329,11 @@ struct PassBLane {
         const R rf = a.rho_factor ? rho_i : R(1);
         // (u~ - u) = dr / dt by the reciprocal the time-step kernel stores
         const R idt = (R)a.dt[1];
-        const R tvf = sizeof(R) == 8 ? -mad2(a.drx[i] * idt, fax, a.dry[i] * idt, fay)
-                                     : -(a.drx[i] * idt * fax + a.dry[i] * idt * fay);
+        R tvf;
+        if constexpr (L64)
+            tvf = -mad2(a.drx[i] * idt, fax, a.dry[i] * idt, fay);
+        else
+            tvf = -(a.drx[i] * idt * fax + a.dry[i] * idt * fay);
         const R half_ac = R(0.5) * (R)a.alpha_e * (R)a.cs;
         const R four_nu = R(4) * (R)a.nu;
         const R dpdt = ((R)a.rho0 * (R)a.cs * (R)a.cs / beta_i) * div +
@@ -326,9 +351,9 @@ struct PassBLane {
 
 // Pass A over the list entries [b, e) of particle i, in list order (team
 // lane t takes entries b + t, b + t + T, ...).
-template <typename R, int T>
+template <typename R, int T, bool LEAN>
 __device__ __forceinline__ void pass_a_list(const PassAArgs<R> &a, int i,
-                                            PassALane<R> &L, const Team<T> &tm,
+                                            PassALane<R, LEAN> &L, const Team<T> &tm,
                                             uint32_t b, uint32_t e) {
     Sep<R> sp;
     sp.init(a.d, a.x, a.y, a.pk, i);
@@ -387,9 +412,9 @@ __device__ __forceinline__ void pass_a_list(const PassAArgs<R> &a, int i,
 }
 
 // Pass B over the list entries [b, e) of particle i, in list order.
-template <typename R, int T>
+template <typename R, int T, bool LEAN>
 __device__ __forceinline__ void pass_b_list(const PassBArgs<R> &a, int i,
-                                            PassBLane<R> &L, const Team<T> &tm,
+                                            PassBLane<R, LEAN> &L, const Team<T> &tm,
                                             uint32_t b, uint32_t e) {
     Sep<R> sp;
     sp.init(a.d, a.x, a.y, a.pk, i);

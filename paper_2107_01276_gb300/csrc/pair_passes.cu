@@ -40,13 +40,14 @@ constexpr int pass_blocks(int lane1) {
 // Pass A of particle i over its list (arithmetic in PassALane): a team of T
 // threads shares particle i.  WALLS = false: a set without wall particles,
 // compiled without the wall loop (whose registers made the one-lane pass B
-// spill at the eight-block bound).
-template <typename R, int T, bool WALLS = true>
+// spill at the eight-block bound) and, on the FP64 path, with the LEAN
+// arithmetic (kernels.cuh).
+template <typename R, int T, bool WALLS>
 __device__ __forceinline__ void pass_a_at(const PassAArgs<R> &a, int i,
                                           const Team<T> &tm) {
-    PassALane<R> L;
+    PassALane<R, !WALLS> L;
     L.init(a, i);
-    pass_a_list<R, T>(a, i, L, tm, a.off[i], a.off[i + 1]);
+    pass_a_list<R, T, !WALLS>(a, i, L, tm, a.off[i], a.off[i + 1]);
     if constexpr (WALLS) L.walls(a, i, tm);
     L.finish(a, i, tm);
 }
@@ -65,10 +66,10 @@ __global__ void __launch_bounds__(128, (pass_blocks<R, T>(PASS_A_BLOCKS)))
 // (float, one lane per particle: at most 64 registers, eight 128-thread
 // blocks per SM, measured faster than six at 80 registers on the graded
 // 1:250 strip)
-template <typename R, int T, bool WALLS = true>
+template <typename R, int T, bool WALLS>
 __device__ __forceinline__ void pass_b_at(const PassBArgs<R> &a, int i,
                                           const Team<T> &tm) {
-    PassBLane<R> L;
+    PassBLane<R, !WALLS> L;
     if (!L.init(a, i)) {
         if (tm.lane == 0) {
             a.dpdt[i] = R(0);
@@ -77,7 +78,7 @@ __device__ __forceinline__ void pass_b_at(const PassBArgs<R> &a, int i,
         }
         return;
     }
-    pass_b_list<R, T>(a, i, L, tm, a.off[i], a.off[i + 1]);
+    pass_b_list<R, T, !WALLS>(a, i, L, tm, a.off[i], a.off[i + 1]);
     if constexpr (WALLS) L.walls(a, i, tm);
     L.finish(a, i, tm, true);
 }
@@ -420,7 +421,11 @@ __global__ void __launch_bounds__(BATCH_THREADS)
         const int q = sp.find(item);
         const PassAArgs<R> &a = args[q];
         const int i = (item - __ldg(&sp.first[q])) * batch_rows(T) + (int)threadIdx.x / T;
-        if (i < a.n) pass_a_at<R, T>(a, i, tm);
+        if (i >= a.n) continue;
+        if (sizeof(R) == 4 || a.w.n > 0)
+            pass_a_at<R, T, true>(a, i, tm);
+        else
+            pass_a_at<R, T, false>(a, i, tm);
     }
 }
 
@@ -432,7 +437,11 @@ __global__ void __launch_bounds__(BATCH_THREADS, sizeof(R) == 4 ? 5 : 1)
         const int q = sp.find(item);
         const PassBArgs<R> &a = args[q];
         const int i = (item - __ldg(&sp.first[q])) * batch_rows(T) + (int)threadIdx.x / T;
-        if (i < a.n) pass_b_at<R, T>(a, i, tm);
+        if (i >= a.n) continue;
+        if (sizeof(R) == 4 || a.w.n > 0)
+            pass_b_at<R, T, true>(a, i, tm);
+        else
+            pass_b_at<R, T, false>(a, i, tm);
     }
 }
 
