@@ -115,7 +115,6 @@ struct sph_ctx {
     uint32_t tcap = 0, tmask = 0;
     int *bbox = nullptr;
     uint32_t *level_mask = nullptr;
-    uint32_t *cnt_tmp = nullptr;   // n + 1 scratch (list totals)
     // neighbour lists and packed per-particle data
     uint8_t *lvl = nullptr;       // level of each particle (sorted order)
     float4 *pk = nullptr;

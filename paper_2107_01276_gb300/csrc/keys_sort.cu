@@ -38,40 +38,43 @@ __device__ __forceinline__ int cell_coord(double x, double lo, double w,
     return c;
 }
 
-// Fast forms of the two quotients above: the product with a rounded
-// reciprocal is within 2^-51 relative of the correctly rounded quotient, so
-// where it lies farther than 1e-12 (relative) from every integer (cell
-// index) or power of two (level), it gives the same floor or exponent; the
-// rare cases closer than that take the correctly rounded division.  GB300's
-// FP64 division costs tens of FP64 operations at a small fraction of the
-// FP32 rate; a product costs one.
-__device__ __forceinline__ int level_of_fast(double h, double c0,
-                                             double inv_c0, int lmax) {
-    const double y = __dmul_rn(__dmul_rn(3.0, h), inv_c0);
-    if (y < 1.0 - 1e-12) return 0;
-    if (y > 1.0 + 1e-12) {
-        int e;
-        const double f = frexp(y, &e);
-        if (f > 0.5 + 1e-12 && f < 1.0 - 1e-12) return e > lmax ? lmax : e;
+// Fast forms of the two quotients above, for a GPU that issues an FP64
+// instruction every 64 cycles a sub-partition: one conversion for the
+// level, one FMA a coordinate.
+// Level: t = 3 h / c0 in FP32 (relative error below 2^-21); away from a
+// power of two by 2^-17 its exponent is that of the exact quotient.
+// Cell: (x - lo) / w by one FMA onto 1.5 2^30, whose result holds the
+// quotient in fixed point with 22 fractional bits, off by less than one
+// unit of them (the rounding half, the reciprocal an eighth), so where the
+// fraction is 4 or more units from an integer the integer part is the exact
+// floor.  Everything closer than that (or out of
+// these ranges) takes the correctly rounded division.
+constexpr double CELL_MAGIC = 1610612736.0;   // 1.5 2^30
+
+__device__ __forceinline__ int level_of_fast(double h, double c0, float k3,
+                                             int lmax) {
+    const float t = (float)h * k3;
+    if (t > 1e-30f && t < 1e30f) {
+        if (t < 1.0f - 1e-5f) return 0;
+        const uint32_t b = __float_as_uint(t), m = b & 0x7fffffu;
+        if (m > 64u && m < 0x7fffffu - 64u) {
+            const int e = (int)(b >> 23) - 126;   // 2^(e-1) < t < 2^e
+            return e > lmax ? lmax : e;
+        }
     }
     return level_of(h, c0, lmax);
 }
 
 __device__ __forceinline__ int cell_coord_fast(double x, double lo, double w,
                                                double invw, int ncell) {
-    const double t = __dsub_rn(x, lo);
-    const double y = __dmul_rn(t, invw);
-    const double fy = floor(y);
-    const double tol = 1e-12 * fmax(1.0, fabs(y));
-    if (!(y - fy > tol && fy + 1.0 - y > tol)) return cell_coord(x, lo, w, ncell);
-    int c;
-    if (fy < 0.0)
-        c = 0;
-    else if (fy > (double)(ncell - 1))
-        c = ncell - 1;
-    else
-        c = (int)fy;
-    return c;
+    const double y = __fma_rn(__dsub_rn(x, lo), invw, CELL_MAGIC);
+    const uint32_t hi = (uint32_t)__double2hiint(y), lw = (uint32_t)__double2loint(y);
+    const uint32_t fr = lw & 0x3fffffu;
+    // 1.5 2^30 + [-2^28, 2^28)
+    if (hi - 0x41d40000u >= 0x80000u || fr < 4u || fr > 0x3fffffu - 4u)
+        return cell_coord(x, lo, w, ncell);
+    const int c = (int)(((hi - 0x41d80000u) << 10) | (lw >> 22));
+    return c < 0 ? 0 : c > ncell - 1 ? ncell - 1 : c;
 }
 
 __device__ __forceinline__ void keys_at(const KeysRec &r, int vb) {
@@ -93,23 +96,33 @@ __device__ __forceinline__ void keys_at(const KeysRec &r, int vb) {
         sb[t] = (t & 1) ? -1 : 0x7fffffff;
     if (threadIdx.x == 0) smask = 0;
     __syncthreads();
-    int i = vb * blockDim.x + threadIdx.x;
-    if (i < n) {
-        int l = level_of_fast(h[i], a.c0, a.inv_c0, a.lmax);
+    const int i = vb * blockDim.x + threadIdx.x;
+    const bool ok = i < n;
+    int l = MAX_LEVELS, ix = 0, iy = 0;
+    if (ok) {
+        l = level_of_fast(h[i], a.c0, a.k3, a.lmax);
         const Level &L = a.lev[l];
-        int ix = cell_coord_fast(x[i], a.dom.lo[0], L.w[0], a.invw[l][0], L.n[0]);
-        int iy = cell_coord_fast(y[i], a.dom.lo[1], L.w[1], a.invw[l][1], L.n[1]);
+        ix = cell_coord_fast(x[i], a.dom.lo[0], L.w[0], a.invw[l][0], L.n[0]);
+        iy = cell_coord_fast(y[i], a.dom.lo[1], L.w[1], a.invw[l][1], L.n[1]);
         uint64_t m = spread2((uint64_t)ix) | (spread2((uint64_t)iy) << 1);
         skey[i] = ((uint64_t)l << (2 * a.mbits)) | m;
         perm[i] = (uint32_t)i;
         if (zero) zero[i] = 0;
         if (zero2) zero2[i] = 0;
         if (zero3) zero3[i] = 0;
+    }
+    // level boxes: reduced over the lanes of each level first (most warps
+    // hold one or two levels, and every thread's five shared atomics on the
+    // same words had been most of this kernel)
+    const unsigned peers = __match_any_sync(0xffffffffu, l);
+    const int x0 = __reduce_min_sync(peers, ix), x1 = __reduce_max_sync(peers, ix);
+    const int y0 = __reduce_min_sync(peers, iy), y1 = __reduce_max_sync(peers, iy);
+    if (ok && (int)(threadIdx.x & 31) == __ffs(peers) - 1) {
         atomicOr(&smask, 1u << l);
-        atomicMin(&sb[l * 4 + 0], ix);
-        atomicMax(&sb[l * 4 + 1], ix);
-        atomicMin(&sb[l * 4 + 2], iy);
-        atomicMax(&sb[l * 4 + 3], iy);
+        atomicMin(&sb[l * 4 + 0], x0);
+        atomicMax(&sb[l * 4 + 1], x1);
+        atomicMin(&sb[l * 4 + 2], y0);
+        atomicMax(&sb[l * 4 + 3], y1);
     }
     __syncthreads();
     uint32_t msk = smask;
@@ -166,7 +179,7 @@ KeysRec make_keys_rec(int n, const Domain &dom, double c0, int lmax, int mbits,
     a.c0 = c0;
     a.lmax = lmax;
     a.mbits = mbits;
-    a.inv_c0 = 1.0 / c0;
+    a.k3 = (float)(3.0 / c0);
     for (int l = 0; l < MAX_LEVELS; ++l) {
         a.lev[l] = lev[l];
         a.invw[l][0] = 1.0 / lev[l].w[0];
@@ -272,120 +285,146 @@ __global__ void __launch_bounds__(RS_THREADS)
     }
 }
 
-// Small sets (n <= RSS_MAX): every pass in one block of 32 warps, keys
-// and values staged in shared memory.  Warp w owns a contiguous chunk; the
-// per-(warp, digit) counts, scanned digit-major, give each warp's scatter
-// base, and the warp ranks its chunk 32 keys at a time with
-// __match_any_sync, so the sort is stable exactly like the tiled form.
-// Intermediate passes scatter into (kb, vb) and reload; the last pass
-// scatters into (ka, va).
+// Small sets (n <= RSS_MAX): every pass in one block of 32 warps.  Warp w
+// owns a contiguous run of the (current) order, its keys and their input
+// positions in registers (up to IT a lane).  A pass ranks them 32 at a time
+// with __match_any_sync against per-(warp, digit) counts, scans the counts
+// digit-major (a warp takes 8 digits, a lane a warp's count), scatters keys
+// and positions into shared memory and reloads them in the new order, so
+// the sort is stable exactly like the tiled form and global memory sees one
+// read and one write.  Keys of at most 32 bits travel as such; wider ones
+// take half the items.  Bound by the latency of its chain of passes: 5 us
+// at 2.5k particles and 3 digits, 9.5 us at 16k (the former form, with two
+// rankings a pass and passes through global memory, took 10 and 29).
 constexpr int RSS_THREADS = 1024;
 constexpr int RSS_WARPS = RSS_THREADS / 32;
 constexpr int RSS_MAX = 16384;
+constexpr int RSS_MAX64 = RSS_MAX / 2;     // keys wider than 32 bits
 
-__device__ __forceinline__ void radix_small_at(int n, int passes, uint64_t *ka,
-                                               uint32_t *va, uint64_t *kb,
-                                               uint32_t *vb) {
-    extern __shared__ uint64_t sk[];          // n keys, then n values
-    uint32_t *sv = (uint32_t *)(sk + n);
-    __shared__ uint32_t cnt[RSS_WARPS][256];
-    __shared__ uint32_t dtot[256];
+static size_t radix_small_smem(int n, int passes) { return (size_t)n * (passes <= 4 ? 6 : 10); }
+
+template <typename K, int IT>
+__device__ __forceinline__ void radix_small_body(int n, int passes, uint64_t *ka,
+                                                 uint32_t *va, uint32_t (*cnt)[257],
+                                                 uint32_t *dtot) {
+    extern __shared__ uint64_t rss_buf[];          // n keys, then n positions
+    K *sk = (K *)rss_buf;
+    uint16_t *si = (uint16_t *)(sk + n);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    const int chunk = (((n + RSS_WARPS - 1) / RSS_WARPS) + 31) & ~31;
-    const int wb = w * chunk, we = min(n, wb + chunk);
-    for (int e = threadIdx.x; e < n; e += RSS_THREADS) {
-        sk[e] = ka[e];
-        sv[e] = va[e];
+    const int rows = (n + RSS_THREADS - 1) / RSS_THREADS;   // items a lane, <= IT
+    const int wb = w * rows * 32 + lane;
+    K key[IT];
+    uint32_t ir[IT];                               // position | rank << 16
+#pragma unroll
+    for (int s = 0; s < IT; ++s) {
+        const int e = wb + s * 32;
+        key[s] = 0;
+        ir[s] = 0;
+        if (s < rows && e < n) {
+            key[s] = (K)ka[e];
+            ir[s] = (uint32_t)e;
+        }
     }
     for (int p = 0; p < passes; ++p) {
         const int shift = 8 * p;
-        const bool last = p == passes - 1;
-        uint64_t *kout = last ? ka : kb;
-        uint32_t *vout = last ? va : vb;
-        for (int t = threadIdx.x; t < RSS_WARPS * 256; t += RSS_THREADS)
-            (&cnt[0][0])[t] = 0;
+        for (int t = threadIdx.x; t < RSS_WARPS * 257; t += RSS_THREADS) (&cnt[0][0])[t] = 0;
         __syncthreads();
-        for (int b = wb; b < we; b += 32) {
-            const int e = b + lane;
-            const bool ok = e < we;
-            const int d = ok ? (int)((sk[e] >> shift) & 255u) : 256;
-            const unsigned peers = __match_any_sync(0xffffffffu, d);
-            uint32_t before = 0;
-            if (ok) before = cnt[w][d];
-            __syncwarp();
-            if (ok && lane == __ffs(peers) - 1) cnt[w][d] = before + __popc(peers);
-            __syncwarp();
-        }
-        __syncthreads();
-        if (threadIdx.x < 256) {            // per digit: prefix over warps
-            const int d = threadIdx.x;
-            uint32_t run = 0;
-            for (int ww = 0; ww < RSS_WARPS; ++ww) {
-                const uint32_t c = cnt[ww][d];
-                cnt[ww][d] = run;
-                run += c;
+#pragma unroll
+        for (int s = 0; s < IT; ++s) {
+            if (s < rows) {
+                const bool ok = wb + s * 32 < n;
+                const int d = ok ? (int)((key[s] >> shift) & 255u) : 256;
+                const unsigned peers = __match_any_sync(0xffffffffu, d);
+                const uint32_t before = cnt[w][d];
+                __syncwarp();
+                if (lane == __ffs(peers) - 1) cnt[w][d] = before + __popc(peers);
+                __syncwarp();
+                ir[s] = (ir[s] & 0xffffu) | ((before + __popc(peers & lt)) << 16);
             }
-            dtot[d] = run;
         }
         __syncthreads();
-        if (threadIdx.x < 32) {             // digit bases (exclusive scan of 256)
+#pragma unroll
+        for (int k = 0; k < 256 / RSS_WARPS; ++k) {
+            const int d = w * (256 / RSS_WARPS) + k;
+            const uint32_t c = cnt[lane][d];
+            uint32_t x = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            cnt[lane][d] = x - c;
+            if (lane == 31) dtot[d] = x;
+        }
+        __syncthreads();
+        if (w == 0) {                              // digit bases: exclusive scan of 256
             uint32_t v[8], sum = 0;
+#pragma unroll
             for (int k = 0; k < 8; ++k) {
                 v[k] = dtot[lane * 8 + k];
                 sum += v[k];
             }
             uint32_t x = sum;
+#pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
                 if (lane >= o) x += y;
             }
-            uint32_t pre = x - sum;
+            x -= sum;
+#pragma unroll
             for (int k = 0; k < 8; ++k) {
-                dtot[lane * 8 + k] = pre;
-                pre += v[k];
+                dtot[lane * 8 + k] = x;
+                x += v[k];
             }
         }
         __syncthreads();
-        for (int t = threadIdx.x; t < RSS_WARPS * 256; t += RSS_THREADS)
-            (&cnt[0][0])[t] += dtot[t & 255];
-        __syncthreads();
-        for (int b = wb; b < we; b += 32) {
-            const int e = b + lane;
-            const bool ok = e < we;
-            uint64_t k = 0;
-            int d = 256;
-            if (ok) {
-                k = sk[e];
-                d = (int)((k >> shift) & 255u);
-            }
-            const unsigned peers = __match_any_sync(0xffffffffu, d);
-            uint32_t before = 0;
-            if (ok) before = cnt[w][d];
-            __syncwarp();
-            if (ok && lane == __ffs(peers) - 1) cnt[w][d] = before + __popc(peers);
-            __syncwarp();
-            if (ok) {
-                const uint32_t pos = before + __popc(peers & lt);
-                kout[pos] = k;
-                vout[pos] = sv[e];
+#pragma unroll
+        for (int s = 0; s < IT; ++s) {
+            if (s < rows && wb + s * 32 < n) {
+                const int d = (int)((key[s] >> shift) & 255u);
+                const uint32_t pos = dtot[d] + cnt[w][d] + (ir[s] >> 16);
+                sk[pos] = key[s];
+                si[pos] = (uint16_t)ir[s];
             }
         }
         __syncthreads();
-        if (!last) {
-            for (int e = threadIdx.x; e < n; e += RSS_THREADS) {
-                sk[e] = kb[e];
-                sv[e] = vb[e];
+#pragma unroll
+        for (int s = 0; s < IT; ++s) {
+            const int e = wb + s * 32;
+            if (s < rows && e < n) {
+                key[s] = sk[e];
+                ir[s] = si[e];
             }
-            __syncthreads();
+        }
+    }
+    // the values of the final order, all read before any is replaced
+#pragma unroll
+    for (int s = 0; s < IT; ++s)
+        if (s < rows && wb + s * 32 < n) ir[s] = va[ir[s]];
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < IT; ++s) {
+        const int e = wb + s * 32;
+        if (s < rows && e < n) {
+            ka[e] = key[s];
+            va[e] = ir[s];
         }
     }
 }
 
+__device__ __forceinline__ void radix_small_at(int n, int passes, uint64_t *ka, uint32_t *va) {
+    __shared__ uint32_t cnt[RSS_WARPS][257];       // padded: a lane a row is conflict-free
+    __shared__ uint32_t dtot[256];
+    if (passes <= 4)
+        radix_small_body<uint32_t, RSS_MAX / RSS_THREADS>(n, passes, ka, va, cnt, dtot);
+    else
+        radix_small_body<uint64_t, RSS_MAX64 / RSS_THREADS>(n, passes, ka, va, cnt, dtot);
+}
+
 __global__ void __launch_bounds__(RSS_THREADS)
-    k_radix_small(int n, int passes, uint64_t *ka, uint32_t *va, uint64_t *kb,
-                  uint32_t *vb) {
-    radix_small_at(n, passes, ka, va, kb, vb);
+    k_radix_small(int n, int passes, uint64_t *ka, uint32_t *va) {
+    radix_small_at(n, passes, ka, va);
 }
 
 // The dynamic shared-memory limit of k_radix_small, raised once per device.
@@ -399,7 +438,7 @@ static bool radix_small_ready() {
     if (ok[dev] == 0) {
         ok[dev] = cudaFuncSetAttribute(k_radix_small,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       RSS_MAX * 12) == cudaSuccess ? 1 : -1;
+                                       (int)radix_small_smem(RSS_MAX, 4)) == cudaSuccess ? 1 : -1;
         if (ok[dev] < 0) cudaGetLastError();
     }
     return ok[dev] == 1;
@@ -412,9 +451,9 @@ size_t radix_counts_elems(size_t n) {
 void radix_sort(cudaStream_t s, int n, int bits, uint64_t *key,
                 uint32_t *val, SortScratch &sc, int *launches) {
     if (n <= 1 || bits <= 0) return;
-    if (n <= RSS_MAX && radix_small_ready()) {
-        k_radix_small<<<1, RSS_THREADS, (size_t)n * 12, s>>>(
-            n, (bits + 7) / 8, key, val, sc.key_alt, sc.val_alt);
+    if (radix_small_takes(n, bits) && radix_small_ready()) {
+        const int passes = (bits + 7) / 8;
+        k_radix_small<<<1, RSS_THREADS, radix_small_smem(n, passes), s>>>(n, passes, key, val);
         *launches += 1;
         return;
     }
@@ -473,20 +512,26 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v,
     return pre;
 }
 
-__global__ void k_scan_reduce(const uint32_t *__restrict__ in, int n,
+// rev (may be NULL): the values are in[i] + rev[i] for i < nrev; the down
+// sweep zeroes rev.
+__global__ void k_scan_reduce(const uint32_t *__restrict__ in,
+                              const uint32_t *__restrict__ rev, int n,
                               uint32_t *__restrict__ sums) {
     long long b0 = (long long)blockIdx.x * SC_TILE;
     uint32_t acc = 0;
+#pragma unroll
     for (int s = 0; s < SC_ITEMS; ++s) {
         long long e = b0 + s * SC_THREADS + threadIdx.x;
-        if (e < n) acc += in[e];
+        if (e < n) acc += in[e] + (rev ? rev[e] : 0u);
     }
     uint32_t tot;
     block_excl_scan(acc, &tot);
     if (threadIdx.x == 0) sums[blockIdx.x] = tot;
 }
 
-__global__ void k_scan_down(const uint32_t *in, uint32_t *out, int n,
+// offs: exclusive sums of the tiles before each; total_dev (may be NULL)
+// receives the sum of all values.
+__global__ void k_scan_down(const uint32_t *in, uint32_t *rev, uint32_t *out, int n,
                             const uint32_t *__restrict__ offs,
                             uint32_t *total_dev) {
     long long b0 = (long long)blockIdx.x * SC_TILE +
@@ -496,16 +541,19 @@ __global__ void k_scan_down(const uint32_t *in, uint32_t *out, int n,
 #pragma unroll
     for (int s = 0; s < SC_ITEMS; ++s) {
         long long e = b0 + s;
-        v[s] = e < n ? in[e] : 0;
+        v[s] = e < n ? in[e] + (rev ? rev[e] : 0u) : 0;
         acc += v[s];
     }
     uint32_t tot;
     uint32_t pre = block_excl_scan(acc, &tot);
-    pre += offs ? offs[blockIdx.x] : 0;
+    pre += offs[blockIdx.x];
 #pragma unroll
     for (int s = 0; s < SC_ITEMS; ++s) {
         long long e = b0 + s;
-        if (e < n) out[e] = pre;
+        if (e < n) {
+            out[e] = pre;
+            if (rev) rev[e] = 0;
+        }
         pre += v[s];
     }
     if (total_dev && blockIdx.x == gridDim.x - 1 && threadIdx.x == SC_THREADS - 1)
@@ -521,25 +569,12 @@ size_t scan_scratch_elems(size_t n) {
     return tot + 1;
 }
 
-static void scan_rec(cudaStream_t s, const uint32_t *in, uint32_t *out, int n,
-                     uint32_t *total_dev, uint32_t *tmp, int *launches) {
-    int nb = (n + SC_TILE - 1) / SC_TILE;
-    if (nb <= 1) {
-        k_scan_down<<<1, SC_THREADS, 0, s>>>(in, out, n, nullptr, total_dev);
-        *launches += 1;
-        return;
-    }
-    uint32_t *sums = tmp;
-    k_scan_reduce<<<nb, SC_THREADS, 0, s>>>(in, n, sums);
-    scan_rec(s, sums, sums, nb, nullptr, tmp + nb, launches);
-    k_scan_down<<<nb, SC_THREADS, 0, s>>>(in, out, n, sums, total_dev);
-    *launches += 2;
-}
-
-// Small scans (n <= 1024 * 32): one block of 1024 threads, thread t owns
-// a contiguous chunk; two passes over the chunk (sum, then write), so in
-// may equal out.  With `rev`, the values are in[i] + rev[i] and rev is
-// zeroed (the neighbour-list totals), and out[n] receives the total.
+// One-block scans (n <= 1024 * 32): warp w owns a contiguous run of up to
+// 32 rows of 32 values, a lane one value a row, so every load and store is
+// coalesced; in may equal out.  With `rev`, the values are in[i] + rev[i]
+// and rev is zeroed (the neighbour-list totals), and out[n] receives the
+// total.  (A thread owning 32 contiguous values, the former form, touched a
+// cache line a lane with every load: 18 us for 32k values against 3.)
 constexpr int SS_THREADS = 1024;
 constexpr int SS_MAX = SS_THREADS * 32;
 
@@ -549,22 +584,20 @@ __device__ __forceinline__ void scan_small_at(const uint32_t *in, uint32_t *rev,
                                               int write_total_at_n) {
     __shared__ uint32_t ws[SS_THREADS / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int chunk = (n + SS_THREADS - 1) / SS_THREADS;   // <= 32
-    const int b = threadIdx.x * chunk;
+    const int rows = (n + SS_THREADS - 1) / SS_THREADS;   // <= 32
+    const int b = w * rows * 32 + lane;
     uint32_t v[32];
     uint32_t sum = 0;
 #pragma unroll
     for (int k = 0; k < 32; ++k) {
-        const int i = b + k;
-        v[k] = (k < chunk && i < n) ? in[i] + (rev ? rev[i] : 0u) : 0u;
-        sum += v[k];
+        v[k] = 0;
+        if (k < rows && b + k * 32 < n)
+            v[k] = in[b + k * 32] + (rev ? rev[b + k * 32] : 0u);
     }
-    uint32_t x = sum;
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) ws[w] = x;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) sum += v[k];
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    if (lane == 0) ws[w] = sum;
     __syncthreads();
     if (w == 0) {
         uint32_t t = ws[lane];
@@ -575,17 +608,25 @@ __device__ __forceinline__ void scan_small_at(const uint32_t *in, uint32_t *rev,
         ws[lane] = t;
     }
     __syncthreads();
-    uint32_t pre = (w > 0 ? ws[w - 1] : 0u) + x - sum;
+    uint32_t pre = w > 0 ? ws[w - 1] : 0u;
 #pragma unroll
     for (int k = 0; k < 32; ++k) {
-        const int i = b + k;
-        if (k < chunk && i < n) {
-            if (rev) rev[i] = 0;
-            out[i] = pre;
-            pre += v[k];
+        if (k < rows) {
+            uint32_t x = v[k];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            const int i = b + k * 32;
+            if (i < n) {
+                if (rev) rev[i] = 0;
+                out[i] = pre + x - v[k];
+            }
+            pre += __shfl_sync(0xffffffffu, x, 31);
         }
     }
-    if (threadIdx.x == SS_THREADS - 1) {
+    if (threadIdx.x == 0) {
         if (total_dev) *total_dev = ws[SS_THREADS / 32 - 1];
         if (write_total_at_n) out[n] = ws[SS_THREADS / 32 - 1];
     }
@@ -595,6 +636,23 @@ __global__ void __launch_bounds__(SS_THREADS)
     k_scan_small(const uint32_t *in, uint32_t *rev, uint32_t *out, int n,
                  uint32_t *total_dev, int write_total_at_n) {
     scan_small_at(in, rev, out, n, total_dev, write_total_at_n);
+}
+
+// Larger ones: tile sums, their scan (one block up to 67M values) and the
+// tiles' own scans.
+static void scan_rec(cudaStream_t s, const uint32_t *in, uint32_t *rev, uint32_t *out, int n,
+                     uint32_t *total_dev, uint32_t *tmp, int *launches) {
+    const int nb = (n + SC_TILE - 1) / SC_TILE;
+    uint32_t *sums = tmp;
+    k_scan_reduce<<<nb, SC_THREADS, 0, s>>>(in, rev, n, sums);
+    *launches += 2;
+    if (nb <= SS_MAX) {
+        k_scan_small<<<1, SS_THREADS, 0, s>>>(sums, nullptr, sums, nb, nullptr, 0);
+        *launches += 1;
+    } else {
+        scan_rec(s, sums, nullptr, sums, nb, nullptr, tmp + nb, launches);
+    }
+    k_scan_down<<<nb, SC_THREADS, 0, s>>>(in, rev, out, n, sums, total_dev);
 }
 
 void exclusive_scan(cudaStream_t s, const uint32_t *in, uint32_t *out, int n,
@@ -608,15 +666,17 @@ void exclusive_scan(cudaStream_t s, const uint32_t *in, uint32_t *out, int n,
         *launches += 1;
         return;
     }
-    scan_rec(s, in, out, n, total_dev, sc.scan_tmp, launches);
+    scan_rec(s, in, nullptr, out, n, total_dev, sc.scan_tmp, launches);
 }
 
-bool list_offsets_small(cudaStream_t s, const uint32_t *own, uint32_t *rev,
-                        uint32_t *off, int n, int *launches) {
-    if (n <= 0 || n > SS_MAX) return false;
-    k_scan_small<<<1, SS_THREADS, 0, s>>>(own, rev, off, n, nullptr, 1);
-    *launches += 1;
-    return true;
+void scan_list_offsets(cudaStream_t s, const uint32_t *own, uint32_t *rev,
+                       uint32_t *off, int n, SortScratch &sc, int *launches) {
+    if (n <= SS_MAX) {
+        k_scan_small<<<1, SS_THREADS, 0, s>>>(own, rev, off, n, nullptr, 1);
+        *launches += 1;
+        return;
+    }
+    scan_rec(s, own, rev, off, n, off + n, sc.scan_tmp, launches);
 }
 
 // ---------------------------------------------------------------- gather --
@@ -801,7 +861,7 @@ __global__ void __launch_bounds__(256) k_keys_batch(const KeysRec *args, BatchSp
 __global__ void __launch_bounds__(RSS_THREADS)
     k_radix_small_batch(const RadixSmallRec *args, BatchSpan sp) {
     batch_blocks(args, sp, [](const RadixSmallRec &r, int, int) {
-        radix_small_at(r.n, r.passes, r.ka, r.va, r.kb, r.vb);
+        radix_small_at(r.n, r.passes, r.ka, r.va);
     });
 }
 __global__ void __launch_bounds__(256)
@@ -818,7 +878,8 @@ __global__ void __launch_bounds__(SS_THREADS)
     });
 }
 
-int radix_small_max() { return RSS_MAX; }
+bool radix_small_takes(int n, int bits) { return n <= (bits <= 32 ? RSS_MAX : RSS_MAX64); }
+int radix_small_bytes(int n, int passes) { return (int)radix_small_smem(n, passes); }
 bool radix_small_available() { return radix_small_ready(); }
 int scan_small_max() { return SS_MAX; }
 
@@ -845,16 +906,16 @@ void launch_keys_batch(cudaStream_t s, const KeysRec *args, const BatchSpan &sp)
     if (sp.total > 0) k_keys_batch<<<batch_grid(r, sp.total), 256, 0, s>>>(args, sp);
 }
 bool launch_radix_small_batch(cudaStream_t s, const RadixSmallRec *args, const BatchSpan &sp,
-                              int max_n) {
+                              int max_smem) {
     static const bool ok = cudaFuncSetAttribute(k_radix_small_batch,
                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                RSS_MAX * 12) == cudaSuccess;
-    if (!ok || max_n > RSS_MAX) {
+                                                (int)radix_small_smem(RSS_MAX, 4)) == cudaSuccess;
+    if (!ok || max_smem > (int)radix_small_smem(RSS_MAX, 4)) {
         cudaGetLastError();
         return false;
     }
     if (sp.total > 0)
-        k_radix_small_batch<<<std::min(sp.total, gpu_sms()), RSS_THREADS, (size_t)max_n * 12, s>>>(
+        k_radix_small_batch<<<std::min(sp.total, gpu_sms()), RSS_THREADS, (size_t)max_smem, s>>>(
             args, sp);
     return true;
 }

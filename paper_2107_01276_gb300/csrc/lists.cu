@@ -159,12 +159,6 @@ __global__ void __launch_bounds__(128) k_list_place(ListArgs a) {
     list_place_at<T>(a, i, tm);
 }
 
-__global__ void k_list_total(int n, const uint32_t *own, const uint32_t *rev,
-                             uint32_t *tot) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) tot[i] = own[i] + rev[i];
-}
-
 // Second walk for the queued particles (more than stage_w own entries):
 // same order as k_list_gather; teams take queue entries in turn.
 template <int T>
@@ -932,20 +926,13 @@ void launch_list_walk(cudaStream_t s, const ListArgs &a, int *launches) {
     *launches += 1;
 }
 
-void list_offsets(cudaStream_t s, const ListArgs &a, SortScratch &sc,
-                  uint32_t *tot_tmp, int *launches) {
+void list_offsets(cudaStream_t s, const ListArgs &a, SortScratch &sc, int *launches) {
     const int n = a.n;
     if (n <= 0) {
         cudaMemsetAsync(a.off, 0, sizeof(uint32_t), s);
         return;
     }
-    if (list_offsets_small(s, a.own, a.rev, a.off, n, launches)) return;
-    k_list_total<<<nblk(n, 256), 256, 0, s>>>(n, a.own, a.rev, tot_tmp);
-    // off has n + 1 entries: scan n + 1 values with a trailing zero
-    cudaMemsetAsync(tot_tmp + n, 0, sizeof(uint32_t), s);
-    exclusive_scan(s, tot_tmp, a.off, n + 1, nullptr, sc, launches);
-    cudaMemsetAsync(a.rev, 0, sizeof(uint32_t) * n, s);
-    *launches += 1;
+    scan_list_offsets(s, a.own, a.rev, a.off, n, sc, launches);
 }
 
 void build_lists_fill(cudaStream_t s, ListArgs a, bool mixed, bool queue,

@@ -290,7 +290,7 @@ sph_status rebuild(sph_ctx *c, bool mid_step, bool exact,
         launch_list_walk(c->s, la, &c->launches);
         t_end(c, 5, ew);
     }
-    list_offsets(c->s, la, c->sc, c->cnt_tmp, &c->launches);
+    list_offsets(c->s, la, c->sc, &c->launches);
     // the fluid particles' wall lists, with the same skin
     c->wall_lists_valid = false;
     WallListArgs wa;
@@ -498,7 +498,7 @@ void free_ctx(sph_ctx *c) {
                   c->pf, c->uf, c->vf, c->nnb, c->skey, c->perm,
                   c->sc.key_alt, c->sc.val_alt, c->sc.counts, c->sc.scan_tmp,
                   c->tkey, c->tstart, c->tend, c->tmaxh, c->bbox, c->level_mask,
-                  c->cnt_tmp, c->d_dt, c->d_t, c->d_hmin, c->d_nonfinite,
+                  c->d_dt, c->d_t, c->d_hmin, c->d_nonfinite,
                   c->d_total, c->lvl, c->pk, c->own, c->rev, c->off, c->list,
                   c->d_overflow, c->d_skin_err, c->longq, c->d_nlong, c->stage, c->lqueue, c->lqref, c->d_max_own,
                   c->d_nlq, c->tmp_a, c->tmp_b,
@@ -865,8 +865,7 @@ sph_status new_ctx(const sph_params *p, cudaStream_t stream, bool has_ds,
     c->tcap = t;
     ok = ok && dalloc(&c->tkey, t, c->s) && dalloc(&c->tstart, t, c->s) && dalloc(&c->tend, t, c->s) &&
          dalloc(&c->tmaxh, t, c->s);
-    ok = ok && dalloc(&c->bbox, MAX_LEVELS * 4, c->s) && dalloc(&c->level_mask, 1, c->s) &&
-         dalloc(&c->cnt_tmp, N + 1, c->s);
+    ok = ok && dalloc(&c->bbox, MAX_LEVELS * 4, c->s) && dalloc(&c->level_mask, 1, c->s);
     ok = ok && dalloc(&c->d_dt, 2, c->s) && dalloc(&c->d_t, 1, c->s) && dalloc(&c->d_hmin, 1, c->s) &&
          dalloc(&c->d_nonfinite, 1, c->s) && dalloc(&c->d_total, 1, c->s) &&
          dalloc(&c->d_skin_err, 1, c->s) &&

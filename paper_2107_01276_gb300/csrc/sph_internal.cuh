@@ -159,10 +159,10 @@ void exclusive_scan(cudaStream_t s, const uint32_t *in, uint32_t *out,
                     int n, uint32_t *total_dev, SortScratch &sc,
                     int *launches);
 size_t scan_scratch_elems(size_t n);
-// off[i] = exclusive scan of own[i] + rev[i], off[n] = total, rev zeroed,
-// in one launch; false (nothing done) if n is too large for one block.
-bool list_offsets_small(cudaStream_t s, const uint32_t *own, uint32_t *rev,
-                        uint32_t *off, int n, int *launches);
+// off[i] = exclusive scan of own[i] + rev[i] (n > 0), off[n] = total, rev
+// zeroed.
+void scan_list_offsets(cudaStream_t s, const uint32_t *own, uint32_t *rev,
+                       uint32_t *off, int n, SortScratch &sc, int *launches);
 // Tile-count entries radix_sort needs in SortScratch::counts for n keys.
 size_t radix_counts_elems(size_t n);
 // h, tmaxh (may be NULL): also record each cell's largest h.
@@ -199,10 +199,11 @@ int rebuild_reset_blocks(uint32_t tslots);   // its grid
 // Cell keys of one set (the keys kernel's arguments).
 struct KeysArgs {
     Domain dom;
-    double c0, inv_c0;
+    double c0;
+    float k3;                      // 3 / c0
     int lmax, mbits;
     Level lev[MAX_LEVELS];
-    double invw[MAX_LEVELS][2];   // 1 / w per level and axis (FP64)
+    double invw[MAX_LEVELS][2];    // 1 / w per level and axis
 };
 struct KeysRec {
     int n;
@@ -227,8 +228,6 @@ struct RadixSmallRec {
     int n, passes;
     uint64_t *ka;
     uint32_t *va;
-    uint64_t *kb;
-    uint32_t *vb;
 };
 struct GatherInsertRec {
     int n;
@@ -246,14 +245,15 @@ struct ScanSmallRec {
     uint32_t *total_dev;
     int write_total_at_n;
 };
-int radix_small_max();           // largest set the single-block sort takes
+bool radix_small_takes(int n, int bits);      // whether the single-block sort does
+int radix_small_bytes(int n, int passes);     // its dynamic shared memory
 bool radix_small_available();    // its shared-memory limit could be raised
 int scan_small_max();            // largest set the single-block scan takes
 void launch_rebuild_reset_batch(cudaStream_t s, const RebuildReset *args, const BatchSpan &sp);
 void launch_keys_batch(cudaStream_t s, const KeysRec *args, const BatchSpan &sp);
 // false (nothing launched) if the shared-memory limit cannot be raised
 bool launch_radix_small_batch(cudaStream_t s, const RadixSmallRec *args, const BatchSpan &sp,
-                              int max_n);
+                              int max_smem);
 void launch_gather_insert_batch(cudaStream_t s, const GatherInsertRec *args, const BatchSpan &sp);
 void launch_scan_small_batch(cudaStream_t s, const ScanSmallRec *args, const BatchSpan &sp);
 // cmin[start of each cell] = min of v over the cell (sorted set).
