@@ -316,8 +316,7 @@ __global__ void k_merge_apply(MergeArgs a) {
             ds = __fadd_ru(ds, __double2float_ru(ra));
             if (__fadd_ru(0.5f * __double2float_ru(hm), ds) > a.budget * h0)
                 atomicOr(a.stale, 1);
-            a.pkw[i] = anchor_record(f[S_X][i], f[S_Y][i], hm, a.lo, a.Ad,
-                                     a.invAd, a.an);
+            a.pkw[i] = anchor_record(f[S_X][i], f[S_Y][i], d2f(hm), a.lo, a.Ad, a.an);
         }
     }
     a.h0[i] = h0;

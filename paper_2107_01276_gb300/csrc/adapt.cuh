@@ -62,7 +62,7 @@ struct MergeArgs {
     float budget;
     int *stale;
     float4 *pkw;                // anchor records, refreshed for merged particles
-    double lo[2], Ad[2], invAd[2];
+    double lo[2], Ad[2];
     // Per particle {m rounded down, m_max rounded up} in FP32, or
     // {+inf, -inf} for a particle that cannot merge (dead, m_max <= 0 or
     // m > m_max): written for every particle in the first round after a

@@ -373,7 +373,6 @@ static void merge_issue(AdaptJob &j) {
     for (int ax = 0; ax < 2; ++ax) {
         a.lo[ax] = c->dom.lo[ax];
         a.Ad[ax] = c->anchor_A[ax];
-        a.invAd[ax] = 1.0 / c->anchor_A[ax];
     }
     j.first = false;
     launch_merge(c->s, a);
@@ -403,11 +402,11 @@ static void finish_issue(AdaptJob &j) {
         if ((st = rebuild(c, false, true, 1.0f + ns / 6.0f + 0.01f)) != SPH_OK)
             return adapt_stop(j, st);
         for (int r = 0; r < ns; ++r) {
-            if (r > 0) pack(c, false);
+            if (r > 0) pack(c);
             launch_shift_round(c->s, shift_args(c), is_mixed(c));
             c->launches += 3;
         }
-        if (ns > 0) pack(c, false);
+        if (ns > 0) pack(c);
         ShiftArgs ha = shift_args(c);
         ha.filter = 1;
         launch_h_update(c->s, ha, is_mixed(c));

@@ -216,8 +216,9 @@ int bits_for(long long v);
 Grid make_grid(const sph_ctx *c);
 Grid grid_for_kernels(const sph_ctx *c);
 ListArgs list_args(sph_ctx *c);
-PackArgs pack_args(sph_ctx *c, bool table_end);
-void pack(sph_ctx *c, bool table_end);
+PackArgs pack_args(sph_ctx *c);
+void pack(sph_ctx *c);
+GatherPackRec gather_pack_rec(sph_ctx *c, bool mid_step);
 bool want_wall_lists(const sph_ctx *c);
 sph_status rebuild(sph_ctx *c, bool mid_step, bool exact = true,
                           float skin = 1.0f, bool for_walls = true);
@@ -370,37 +371,69 @@ inline PassBArgs<R> pass_b_args(sph_ctx *c, const PassAArgs<R> &a) {
     return b;
 }
 
+// Between the stages of a step the predicted state and the start's trade
+// places: f[F_X] .. f[F_P] hold the one the next evaluation reads, f[F_X0]
+// .. f[F_P0] the other (and so their gather targets).  Called after the
+// predictor and again after the corrector.
+inline void swap_stage(sph_ctx *c) {
+    for (int k = 0; k < 5; ++k) {
+        std::swap(c->f[F_X + k], c->f[F_X0 + k]);
+        std::swap(c->falt[F_X + k], c->falt[F_X0 + k]);
+    }
+}
+
+// The stage's arguments: the predictor (f < 1) takes the state in f[F_X] ..
+// f[F_P] to f[F_X0] .. f[F_P0]; after swap_stage the corrector updates the
+// start's buffers in place.  fuse: the mixed predictor also writes the
+// records of the predicted state and the corrector the density (false: the
+// caller runs the packing and the density store).
 template <typename R>
-inline PecArgs<R> pec_args(sph_ctx *c, double f) {
+inline PecArgs<R> pec_args(sph_ctx *c, double f, bool fuse) {
     PecArgs<R> a;
+    const bool predict = f < 1.0, mixed = sizeof(R) == sizeof(float);
+    const int in = predict ? F_X : F_X0;
     a.n = c->n;
     a.d = c->dom;
     a.f = f;
-    a.save = f < 1.0 ? 1 : 0;   // the predictor starts the step: keep x0..p0
     a.h = c->f[F_H];
     // with skin lists, the predictor's moves must stay within the skin: a
     // pair approaches by at most 2 disp_lim max(h) <= (skin - 1) 3 max(h)
     a.disp_lim = 1.5 * ((double)c->skin - 1.0);
-    a.skin_err = (a.save && c->skin > 1.0f) ? c->d_skin_err : nullptr;
+    a.skin_err = (predict && c->skin > 1.0f) ? c->d_skin_err : nullptr;
     a.dt = c->d_dt;
-    a.sponge_w = c->prm.sponge_width > 0 && f >= 1.0 ? c->prm.sponge_width : 0.0;
+    a.sponge_w = c->prm.sponge_width > 0 && !predict ? c->prm.sponge_width : 0.0;
     a.sponge_x1 = c->dom.lo[0] + c->prm.sponge_width;
     a.sponge_U = c->prm.U_ref;
-    a.x0 = c->f[F_X0];
-    a.y0 = c->f[F_Y0];
-    a.u0 = c->f[F_U0];
-    a.v0 = c->f[F_V0];
-    a.p0 = c->f[F_P0];
+    a.x0 = c->f[in];
+    a.y0 = c->f[in + 1];
+    a.u0 = c->f[in + 2];
+    a.v0 = c->f[in + 3];
+    a.p0 = c->f[in + 4];
     a.dudt = (const R *)c->dudt;
     a.dvdt = (const R *)c->dvdt;
     a.dpdt = (const R *)c->dpdt;
     a.drx = (const R *)c->drx;
     a.dry = (const R *)c->dry;
-    a.x = c->f[F_X];
-    a.y = c->f[F_Y];
-    a.u = c->f[F_U];
-    a.v = c->f[F_V];
-    a.p = c->f[F_P];
+    a.x = c->f[F_X0];
+    a.y = c->f[F_Y0];
+    // (the wall condition reads the predicted u, v, p in FP64, and the
+    // FP64 path's mid-step build carries them)
+    const bool uvp = !predict || !mixed || !fuse || c->wall.n > 0;
+    a.u = uvp ? c->f[F_U0] : nullptr;
+    a.v = uvp ? c->f[F_V0] : nullptr;
+    a.p = uvp ? c->f[F_P0] : nullptr;
+    a.pk = predict && mixed && fuse ? c->pk : nullptr;
+    a.pf = c->pf;
+    a.uf = c->uf;
+    a.vf = c->vf;
+    a.an = c->an;
+    for (int ax = 0; ax < 2; ++ax) {
+        a.lo[ax] = c->dom.lo[ax];
+        a.Ad[ax] = c->anchor_A[ax];
+    }
+    a.rho = (const R *)c->rhoR;
+    a.rho_out = predict || !fuse ? nullptr : c->f[F_RHO];
+    a.walls = c->wall.n > 0 ? 1 : 0;
     return a;
 }
 

@@ -187,7 +187,7 @@ static bool stage_pec(Stager &st, const std::vector<sph_ctx *> &cs, double f,
                       std::vector<PhaseGroup> &g) {
     return stage_phase<PecArgs<R>>(
         st, cs, [](sph_ctx *) { return 1; }, [](sph_ctx *c) { return c->n; },
-        [f](sph_ctx *c) { return pec_args<R>(c, f); }, g);
+        [f](sph_ctx *c) { return pec_args<R>(c, f, false); }, g);
 }
 
 static bool stage_eval(Stager &st, const std::vector<sph_ctx *> &m32,
@@ -251,7 +251,7 @@ static size_t batch_bytes_per_instance() {
     // a batched small-set build (two for FP64 contexts: one mid-step)
     const size_t build = up(sizeof(DtSmallRec)) + up(sizeof(RebuildReset)) +
                          up(sizeof(KeysRec)) + up(sizeof(RadixSmallRec)) +
-                         up(sizeof(GatherInsertRec)) + up(sizeof(PackArgs)) +
+                         up(sizeof(GatherPackRec)) + up(sizeof(PackArgs)) +
                          3 * up(sizeof(ListArgs)) + up(sizeof(ScanSmallRec)) +
                          2 * up(sizeof(SortSegRec));
     return 2 * eval + 2 * build + up(sizeof(PackArgs)) + up(sizeof(RhoStoreArgs));
@@ -294,7 +294,7 @@ struct SmallBuild {
     RebuildReset rr;
     KeysRec keys;
     RadixSmallRec rs;
-    GatherInsertRec gi;
+    GatherPackRec gp;
     PackArgs pack;
     ListArgs la;
     ScanSmallRec scan;
@@ -336,27 +336,8 @@ static void plan_small_build(sph_ctx *c, bool mid_step, float skin, bool with_dt
     B.rs.passes = (2 * c->mbits + c->lbits + 7) / 8;
     B.rs.ka = c->skey;
     B.rs.va = c->perm;
-    GatherList &gl = B.gi.g;
-    memset(&gl, 0, sizeof(gl));
-    const int last = mid_step ? NF : F_X0;
-    for (int k = 0; k < last; ++k) {
-        if (!c->f[k]) continue;
-        gl.src[gl.nd] = c->f[k];
-        gl.dst[gl.nd] = c->falt[k];
-        gl.nd++;
-    }
-    gl.isrc[0] = c->id;
-    gl.idst[0] = c->id_alt;
-    gl.ni = 1;
-    B.gi.n = n;
-    B.gi.perm = c->perm;
-    B.gi.skey = c->skey;
-    B.gi.tkey = c->tkey;
-    B.gi.tstart = c->tstart;
-    B.gi.tmask = c->tmask;
-    for (int k = 0; k < last; ++k) std::swap(c->f[k], c->falt[k]);
-    std::swap(c->id, c->id_alt);
-    B.pack = pack_args(c, true);
+    B.gp = gather_pack_rec(c, mid_step);
+    B.pack = pack_args(c);
     B.la = list_args(c);
     B.la.skin = skin;
     c->skin = skin;
@@ -406,7 +387,7 @@ static bool launch_small_builds(sph_batch *b, Stager &st, const std::vector<Smal
     std::vector<RebuildReset> rr;
     std::vector<KeysRec> keys;
     std::vector<RadixSmallRec> rs;
-    std::vector<GatherInsertRec> gi;
+    std::vector<GatherPackRec> gp;
     std::vector<PackArgs> pk;
     std::vector<ScanSmallRec> sc;
     std::vector<SortSegRec> seg;
@@ -419,7 +400,7 @@ static bool launch_small_builds(sph_batch *b, Stager &st, const std::vector<Smal
         rr.push_back(B.rr);
         keys.push_back(B.keys);
         rs.push_back(B.rs);
-        gi.push_back(B.gi);
+        gp.push_back(B.gp);
         pk.push_back(B.pack);
         sc.push_back(B.scan);
         seg.push_back(B.seg);
@@ -457,12 +438,12 @@ static bool launch_small_builds(sph_batch *b, Stager &st, const std::vector<Smal
         }
         return stage_group(st, la, items, team, g);
     };
-    PhaseGroup gdt, grr, gkeys, grs, ggi, gpk, gsc, gfq, gsr, gsl;
+    PhaseGroup gdt, grr, gkeys, grs, ggp, gpk, gsc, gfq, gsr, gsl;
     std::vector<PhaseGroup> gwalk(walk_teams.size()), gplace(place_teams.size());
     bool ok = true;
     if (with_dt) ok = ok && stage_group(st, dt, i_one, 1, gdt);
     ok = ok && stage_group(st, rr, i_rr, 1, grr) && stage_group(st, keys, i_256, 1, gkeys) &&
-         stage_group(st, rs, i_one, 1, grs) && stage_group(st, gi, i_256, 1, ggi) &&
+         stage_group(st, rs, i_one, 1, grs) && stage_group(st, gp, i_256, 1, ggp) &&
          stage_group(st, pk, i_128, 1, gpk) && stage_group(st, sc, i_one, 1, gsc);
     std::vector<ListArgs> la_all;
     for (const SmallBuild &B : bs) la_all.push_back(B.la);
@@ -494,7 +475,7 @@ static bool launch_small_builds(sph_batch *b, Stager &st, const std::vector<Smal
     if (!launch_radix_small_batch(b->s, (const RadixSmallRec *)(st.d + grs.off_args), sp(grs),
                                   max_smem))
         return false;
-    launch_gather_insert_batch(b->s, (const GatherInsertRec *)(st.d + ggi.off_args), sp(ggi));
+    launch_gather_batch(b->s, (const GatherPackRec *)(st.d + ggp.off_args), sp(ggp));
     launch_pack_batch(b->s, (const PackArgs *)(st.d + gpk.off_args), sp(gpk), b->pack_blocks);
     nl += 5;
     for (size_t u = 0; u < walk_teams.size(); ++u) {
@@ -585,10 +566,15 @@ static sph_status batch_body(sph_batch *b, const std::vector<sph_ctx *> &all,
     EvalStage e1, e2;
     if (!stage_eval(st, m32, m64, all, 0.5, e1))
         return fail(all[0], SPH_ECUDA, "sph_batch_step: staging overflow");
+    for (sph_ctx *c : all) swap_stage(c);
+    auto undo = [&](const char *why) {   // nothing ran
+        for (sph_ctx *c : all) swap_stage(c);
+        return fail(all[0], SPH_ECUDA, why);
+    };
     std::vector<PhaseGroup> gpack, grho;
     bool ok = stage_phase<PackArgs>(
         st, m32, [](sph_ctx *) { return 1; }, [](sph_ctx *c) { return c->n; },
-        [](sph_ctx *c) { return pack_args(c, false); }, gpack);
+        [](sph_ctx *c) { return pack_args(c); }, gpack);
     ok = ok && stage_phase<RhoStoreArgs>(
         st, m32, [](sph_ctx *) { return 1; }, [](sph_ctx *c) { return c->n; },
         [](sph_ctx *c) {
@@ -598,10 +584,10 @@ static sph_status batch_body(sph_batch *b, const std::vector<sph_ctx *> &all,
             a.dst = c->f[F_RHO];
             return a;
         }, grho);
-    if (!ok) return fail(all[0], SPH_ECUDA, "sph_batch_step: staging overflow");
+    if (!ok) return undo("sph_batch_step: staging overflow");
     const bool fp64 = !m64.empty();
     if (!fp64 && !stage_eval(st, m32, m64, all, 1.0, e2))
-        return fail(all[0], SPH_ECUDA, "sph_batch_step: staging overflow");
+        return undo("sph_batch_step: staging overflow");
     st.flush(b->s);
     launch_eval(b, st, e1);
     // 3. mid-step: mixed instances repack at the predicted state (their
@@ -653,6 +639,7 @@ static sph_status batch_body(sph_batch *b, const std::vector<sph_ctx *> &all,
         cudaMemcpyAsync(c->f[F_RHO], c->rhoR, sizeof(double) * c->n, cudaMemcpyDeviceToDevice,
                         b->s);
     for (sph_ctx *c : all) {
+        swap_stage(c);
         c->grid_valid = false;
         c->rhs_valid = true;
         c->steps += 1;

@@ -728,49 +728,6 @@ __global__ void k_table_end(int n, const uint64_t *__restrict__ skey,
     table_mark_end(i, n, skey, tkey, tend, tmask, h, tmaxh);
 }
 
-// Gather in sorted order fused with the insertion of each cell's start.
-__device__ __forceinline__ void gather_insert_at(int i, int n, const uint32_t *__restrict__ perm,
-                                                 const GatherList &g,
-                                                 const uint64_t *__restrict__ skey,
-                                                 uint64_t *tkey, uint32_t *tstart,
-                                                 uint32_t tmask) {
-    if (i >= n) return;
-    uint32_t src = perm[i];
-    if (!SPH_DCHECK(src < (uint32_t)n)) return;
-    for (int k = 0; k < g.nd; ++k) g.dst[k][i] = g.src[k][src];
-    for (int k = 0; k < g.ni; ++k) g.idst[k][i] = g.isrc[k][src];
-    uint64_t k = skey[i];
-    if (i > 0 && skey[i - 1] == k) return;
-    uint32_t slot = hash_slot(k, tmask);
-    for (uint32_t it = 0; it <= tmask; ++it) {
-        unsigned long long prev = atomicCAS((unsigned long long *)&tkey[slot],
-                                            (unsigned long long)EMPTY_KEY,
-                                            (unsigned long long)k);
-        if (prev == EMPTY_KEY || prev == k) {
-            tstart[slot] = (uint32_t)i;
-            return;
-        }
-        slot = (slot + 1) & tmask;
-    }
-}
-
-__global__ void k_gather_insert(int n, const uint32_t *__restrict__ perm,
-                                GatherList g, const uint64_t *__restrict__ skey,
-                                uint64_t *tkey, uint32_t *tstart,
-                                uint32_t tmask) {
-    gather_insert_at(blockIdx.x * blockDim.x + threadIdx.x, n, perm, g, skey, tkey,
-                     tstart, tmask);
-}
-
-void gather_insert(cudaStream_t s, int n, const uint32_t *perm,
-                   const GatherList &g, const uint64_t *skey, uint64_t *tkey,
-                   uint32_t *tstart, uint32_t tmask, int *launches) {
-    if (n <= 0) return;
-    k_gather_insert<<<(n + 255) / 256, 256, 0, s>>>(n, perm, g, skey, tkey,
-                                                     tstart, tmask);
-    *launches += 1;
-}
-
 // Reset before a rebuild: level bounding boxes and mask, every table key,
 // and up to four counters.
 __device__ __forceinline__ void rebuild_reset_at(const RebuildReset &r, uint32_t vb,
@@ -864,13 +821,6 @@ __global__ void __launch_bounds__(RSS_THREADS)
         radix_small_at(r.n, r.passes, r.ka, r.va);
     });
 }
-__global__ void __launch_bounds__(256)
-    k_gather_insert_batch(const GatherInsertRec *args, BatchSpan sp) {
-    batch_blocks(args, sp, [](const GatherInsertRec &r, int vb, int) {
-        gather_insert_at(vb * blockDim.x + threadIdx.x, r.n, r.perm, r.g, r.skey, r.tkey,
-                         r.tstart, r.tmask);
-    });
-}
 __global__ void __launch_bounds__(SS_THREADS)
     k_scan_small_batch(const ScanSmallRec *args, BatchSpan sp) {
     batch_blocks(args, sp, [](const ScanSmallRec &r, int, int) {
@@ -918,10 +868,6 @@ bool launch_radix_small_batch(cudaStream_t s, const RadixSmallRec *args, const B
         k_radix_small_batch<<<std::min(sp.total, gpu_sms()), RSS_THREADS, (size_t)max_smem, s>>>(
             args, sp);
     return true;
-}
-void launch_gather_insert_batch(cudaStream_t s, const GatherInsertRec *args, const BatchSpan &sp) {
-    static const int r = resident(k_gather_insert_batch, 256, 0);
-    if (sp.total > 0) k_gather_insert_batch<<<batch_grid(r, sp.total), 256, 0, s>>>(args, sp);
 }
 void launch_scan_small_batch(cudaStream_t s, const ScanSmallRec *args, const BatchSpan &sp) {
     static const int r = resident(k_scan_small_batch, SS_THREADS, 0);

@@ -9,21 +9,30 @@ namespace sph {
 
 struct PackArgs {
     int n;
-    int lshift;                 // 2 * mbits: level = skey >> lshift
     int mixed;
-    const uint64_t *skey;
     const double *x, *y, *h, *m, *p, *u, *v;
     double lo[2], Ad[2];        // anchor origin and side (FP64)
-    double invAd[2];            // 1 / Ad
     Anchor an;
-    uint8_t *lev;
     float4 *pk;                 // {xl, yl, h, gx | gy << 16}
     float *mf, *pf, *uf, *vf;
-    // cell table: the last particle of each cell records its end
-    const uint64_t *tkey;
-    uint32_t *tend;
+};
+
+// The permutation gather of a rebuild (f[perm[i]] to falt[i]; the first
+// fields of g are x, y, u, v, p, rho, m, h), with everything the sorted
+// order gives at once: levels, anchor records and float mirrors, and the
+// cell table's entries.
+struct GatherPackRec {
+    int n;
+    int lshift;                 // 2 * mbits: level = skey >> lshift
+    const uint32_t *perm;
+    GatherList g;
+    const uint64_t *skey;
+    uint64_t *tkey;
+    uint32_t *tstart, *tend;
     uint32_t tmask;
     float *tmaxh;               // per slot: the cell's largest h
+    uint8_t *lev;
+    PackArgs p;                 // outputs, anchor lattice (inputs unused)
 };
 
 struct ListArgs {
@@ -61,9 +70,12 @@ struct ListArgs {
 };
 
 void launch_pack(cudaStream_t s, const PackArgs &a);
-// packing over the work items of several instances (batched step); blocks:
-// the persistent grid (resident blocks per SM from the function below
-// times the SMs)
+void launch_gather_pack(cudaStream_t s, const GatherPackRec &r, int *launches);
+// over the work items of several instances (batched step): the gather with
+// the levels and the table entries (256-thread items), and the packing;
+// blocks: the persistent grid (resident blocks per SM from the function
+// below times the SMs)
+void launch_gather_batch(cudaStream_t s, const GatherPackRec *args, const BatchSpan &sp);
 void launch_pack_batch(cudaStream_t s, const PackArgs *args, const BatchSpan &sp,
                        int blocks);
 int pack_batch_blocks_per_sm();

@@ -468,27 +468,25 @@ __device__ __forceinline__ void anchor_sep(const Anchor &an, const float4 &pi,
 // lattice; next to a cell edge it may be the neighbouring cell, which only
 // moves the offset to within A / 256 outside [0, A): the separation error
 // bound assumes an offset within about A) and the offset xl = x - lo - g A
-// in FP64 with one rounding, then rounded to FP32.  One FP64 subtraction,
-// one FMA and three conversions a coordinate (FP64 work is slow on this
-// GPU).
-__device__ __forceinline__ float4 anchor_record(double x, double y, double h,
+// in FP64 with one rounding, then rounded to FP32.  One FP64 subtraction
+// and one FMA a coordinate, the conversions on the integer pipe (FP64 work
+// is slow on this GPU).
+__device__ __forceinline__ float4 anchor_record(double x, double y, float h,
                                                 const double *lo,
                                                 const double *A,
-                                                const double *invA,
                                                 const Anchor &an) {
-    (void)invA;
     const double q[2] = {x, y};
     int g[2];
     float xl[2];
 #pragma unroll
     for (int ax = 0; ax < 2; ++ax) {
         const double t = __dsub_rn(q[ax], lo[ax]);
-        const float c = floorf((float)t * an.iA[ax]);
+        const float c = floorf(d2f(t) * an.iA[ax]);
         const int gi = c < 0.0f ? 0 : (c > (float)(an.n[ax] - 1) ? an.n[ax] - 1 : (int)c);
         g[ax] = gi;
-        xl[ax] = (float)__fma_rn(-(double)gi, A[ax], t);
+        xl[ax] = d2f(__fma_rn(-u2d((uint32_t)gi), A[ax], t));
     }
-    return make_float4(xl[0], xl[1], (float)h,
+    return make_float4(xl[0], xl[1], h,
                        __uint_as_float((unsigned)g[0] | ((unsigned)g[1] << 16)));
 }
 

@@ -54,8 +54,6 @@ struct PecArgs {
     int n;
     Domain d;
     double f;                  // 0.5 predict, 1.0 correct
-    int save;                  // 1: the current x, y, u, v, p are the stage
-                               // start; copy them into x0..p0 first
     // with skin_err: a particle moving more than disp_lim h in this stage
     // sets *skin_err (the neighbour lists of the step no longer hold N(i))
     const double *h;
@@ -65,9 +63,21 @@ struct PecArgs {
     // sponge layer (sph_params.sponge_width; corrector only): width (0:
     // off), its downstream edge, the target speed
     double sponge_w, sponge_x1, sponge_U;
-    const double *x0, *y0, *u0, *v0, *p0;
+    const double *x0, *y0, *u0, *v0, *p0;   // state at the step's start
     const R *dudt, *dvdt, *dpdt, *drx, *dry;
+    // the new state; may be the start's buffers (corrector), u, v, p NULL:
+    // not needed in FP64 (the predicted state of a set without walls)
     double *x, *y, *u, *v, *p;
+    // mixed predictor: the anchor records (their h stays) and float mirrors
+    // of the new state, which the second evaluation reads
+    float4 *pk;
+    float *pf, *uf, *vf;
+    Anchor an;
+    double lo[2], Ad[2];
+    // corrector: the summation density into the FP64 state
+    const R *rho;
+    double *rho_out;
+    int walls;                 // the set has walls (see pec_at)
 };
 
 struct ConvList {

@@ -153,15 +153,11 @@ ListArgs list_args(sph_ctx *c) {
 }
 
 // Per-particle anchor records (and the mixed path's float mirrors) at the
-// current positions; with table_end also the cell ends of the table (part
-// of a rebuild).
-PackArgs pack_args(sph_ctx *c, bool table_end) {
-    const int n = c->n;
+// current positions.
+PackArgs pack_args(sph_ctx *c) {
     PackArgs pa;
-    pa.n = n;
-    pa.lshift = 2 * c->mbits;
+    pa.n = c->n;
     pa.mixed = is_mixed(c) ? 1 : 0;
-    pa.skey = c->skey;
     pa.x = c->f[F_X];
     pa.y = c->f[F_Y];
     pa.h = c->f[F_H];
@@ -172,24 +168,50 @@ PackArgs pack_args(sph_ctx *c, bool table_end) {
     for (int ax = 0; ax < 2; ++ax) {
         pa.lo[ax] = c->dom.lo[ax];
         pa.Ad[ax] = c->anchor_A[ax];
-        pa.invAd[ax] = 1.0 / c->anchor_A[ax];
     }
     pa.an = c->an;
-    pa.lev = c->lvl;
     pa.pk = c->pk;
     pa.mf = c->mf;
     pa.pf = c->pf;
     pa.uf = c->uf;
     pa.vf = c->vf;
-    pa.tkey = c->tkey;
-    pa.tend = table_end ? c->tend : nullptr;
-    pa.tmask = c->tmask;
-    pa.tmaxh = c->tmaxh;
     return pa;
 }
-void pack(sph_ctx *c, bool table_end) {
-    launch_pack(c->s, pack_args(c, table_end));
+void pack(sph_ctx *c) {
+    launch_pack(c->s, pack_args(c));
     c->launches += 1;
+}
+
+// The gather of a rebuild, and the swap of the state buffers it fills.
+// mid_step: the start's copies x0..p0 travel too.
+GatherPackRec gather_pack_rec(sph_ctx *c, bool mid_step) {
+    GatherPackRec r;
+    GatherList &gl = r.g;
+    memset(&gl, 0, sizeof(gl));
+    const int last = mid_step ? NF : F_X0;
+    for (int k = 0; k < last; ++k) {
+        if (!c->f[k]) continue;
+        gl.src[gl.nd] = c->f[k];
+        gl.dst[gl.nd] = c->falt[k];
+        gl.nd++;
+    }
+    gl.isrc[0] = c->id;
+    gl.idst[0] = c->id_alt;
+    gl.ni = 1;
+    r.n = c->n;
+    r.lshift = 2 * c->mbits;
+    r.perm = c->perm;
+    r.skey = c->skey;
+    r.tkey = c->tkey;
+    r.tstart = c->tstart;
+    r.tend = c->tend;
+    r.tmask = c->tmask;
+    r.tmaxh = c->tmaxh;
+    r.lev = c->lvl;
+    for (int k = 0; k < last; ++k) std::swap(c->f[k], c->falt[k]);
+    std::swap(c->id, c->id_alt);
+    r.p = pack_args(c);
+    return r;
 }
 
 // exact: read the list total back (one synchronisation) and grow the list
@@ -263,24 +285,8 @@ sph_status rebuild(sph_ctx *c, bool mid_step, bool exact,
     c->launches += 1;
     radix_sort(c->s, n, 2 * c->mbits + c->lbits, c->skey, c->perm, c->sc,
                &c->launches);
-    GatherList gl;
-    memset(&gl, 0, sizeof(gl));
-    int last = mid_step ? NF : F_X0;
-    for (int k = 0; k < last; ++k) {
-        if (!c->f[k]) continue;
-        gl.src[gl.nd] = c->f[k];
-        gl.dst[gl.nd] = c->falt[k];
-        gl.nd++;
-    }
-    gl.isrc[0] = c->id;
-    gl.idst[0] = c->id_alt;
-    gl.ni = 1;
-    gather_insert(c->s, n, c->perm, gl, c->skey, c->tkey, c->tstart, c->tmask,
-                  &c->launches);
+    launch_gather_pack(c->s, gather_pack_rec(c, mid_step), &c->launches);
     t_end(c, 6, es);
-    for (int k = 0; k < last; ++k) std::swap(c->f[k], c->falt[k]);
-    std::swap(c->id, c->id_alt);
-    pack(c, true);
     ListArgs la = list_args(c);
     la.skin = skin;
     c->skin = skin;
@@ -425,7 +431,7 @@ void run_passes(sph_ctx *c) {
 
 template <typename R>
 static void pec(sph_ctx *c, double f) {
-    const PecArgs<R> a = pec_args<R>(c, f);
+    const PecArgs<R> a = pec_args<R>(c, f, true);
     cudaEvent_t ev;
     t_begin(c, 3, &ev);
     launch_pec<R>(c->s, a);
@@ -1019,16 +1025,15 @@ sph_status pec_step(sph_ctx *c, bool exact) {
     sph_status st = rebuild(c, false, exact, step_skin);
     if (st != SPH_OK) return st;
     run_passes(c);
-    run_pec(c, 0.5);
-    if (step_skin > 1.0f) {
-        pack(c, false);   // anchor records and mirrors at the predicted state
-    } else {
+    run_pec(c, 0.5);   // (mixed: and the records of the predicted state)
+    swap_stage(c);
+    if (!(step_skin > 1.0f)) {
         st = rebuild(c, true, false);
         if (st != SPH_OK) return st;
     }
     run_passes(c);
-    run_pec(c, 1.0);
-    store_rho(c);
+    run_pec(c, 1.0);   // and the density into the state
+    swap_stage(c);
     c->grid_valid = false;   // positions moved since the last rebuild
     c->rhs_valid = true;     // rates of the n+1/2 evaluation, current order
     c->steps += 1;

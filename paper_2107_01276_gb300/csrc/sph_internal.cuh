@@ -102,6 +102,47 @@ __host__ __device__ inline uint32_t hash_slot(uint64_t k, uint32_t mask) {
     return (uint32_t)k & mask;
 }
 
+// float <-> double without the FP64 pipe, which issues one instruction every
+// 64 cycles a sub-partition, conversions included.  f2d: exact; a subnormal
+// gives a zero of its sign (the pass kernels flush them anyway).  d2f: round
+// to nearest even for magnitudes a normal float holds, and zero; the rest
+// (subnormal results, overflow, infinities, NaN) take the conversion
+// instruction.
+__device__ __forceinline__ double f2d(float v) {
+    const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
+    uint32_t hi = (m >> 3) + 0x38000000u;
+    if (m >= 0x7f800000u) hi = (m >> 3) | 0x7ff00000u;
+    if (m < 0x00800000u) return __hiloint2double((int)(b & 0x80000000u), 0);
+    return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
+}
+__device__ __forceinline__ float d2f(double v) {
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    const uint32_t m = hi & 0x7fffffffu;
+    if (m - 0x38100000u >= 0x47e00000u - 0x38100000u) {
+        if ((m | lo) == 0u) return __uint_as_float(hi);
+        return (float)v;
+    }
+    uint32_t f = ((m - 0x38000000u) << 3) | (lo >> 29);
+    const uint32_t rem = lo << 3;
+    f += (rem > 0x80000000u || (rem == 0x80000000u && (f & 1u))) ? 1u : 0u;
+    return __uint_as_float(f | (hi & 0x80000000u));
+}
+// unsigned integers below 2^31, exactly
+__device__ __forceinline__ double u2d(uint32_t v) {
+    if (v == 0u) return 0.0;
+    const int z = __clz((int)v);
+    const uint32_t m = v << z;                     // leading one at bit 31
+    return __hiloint2double((int)(((uint32_t)(1054 - z) << 20) + ((m >> 11) & 0xfffffu)),
+                            (int)(m << 21));
+}
+// rounded up, v > 0
+__device__ __forceinline__ float d2f_up(double v) {
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    if (hi - 0x38100000u >= 0x47e00000u - 0x38100000u) return __double2float_ru(v);
+    const uint32_t f = ((hi - 0x38000000u) << 3) | (lo >> 29);
+    return __uint_as_float(f + ((lo << 3) != 0u ? 1u : 0u));
+}
+
 // Minimum-image separation component, FP64, no contraction.  A separation
 // whose high word is below the half period's is already the minimum image
 // (most pairs): that test runs on the integer pipe.
@@ -181,11 +222,6 @@ struct GatherList {
 };
 void gather_by_perm(cudaStream_t s, int n, const uint32_t *perm,
                     const GatherList &g, int *launches);
-// gather_by_perm fused with the insertion of each cell's start into the
-// table (keys reset to EMPTY_KEY beforehand).
-void gather_insert(cudaStream_t s, int n, const uint32_t *perm,
-                   const GatherList &g, const uint64_t *skey, uint64_t *tkey,
-                   uint32_t *tstart, uint32_t tmask, int *launches);
 struct RebuildReset {
     int *bbox;
     uint32_t *level_mask;
@@ -229,15 +265,6 @@ struct RadixSmallRec {
     uint64_t *ka;
     uint32_t *va;
 };
-struct GatherInsertRec {
-    int n;
-    const uint32_t *perm;
-    GatherList g;
-    const uint64_t *skey;
-    uint64_t *tkey;
-    uint32_t *tstart;
-    uint32_t tmask;
-};
 struct ScanSmallRec {
     const uint32_t *in;
     uint32_t *rev, *out;
@@ -254,7 +281,6 @@ void launch_keys_batch(cudaStream_t s, const KeysRec *args, const BatchSpan &sp)
 // false (nothing launched) if the shared-memory limit cannot be raised
 bool launch_radix_small_batch(cudaStream_t s, const RadixSmallRec *args, const BatchSpan &sp,
                               int max_smem);
-void launch_gather_insert_batch(cudaStream_t s, const GatherInsertRec *args, const BatchSpan &sp);
 void launch_scan_small_batch(cudaStream_t s, const ScanSmallRec *args, const BatchSpan &sp);
 // cmin[start of each cell] = min of v over the cell (sorted set).
 void launch_cell_min(cudaStream_t s, int n, const uint64_t *skey,
