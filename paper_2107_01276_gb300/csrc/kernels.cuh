@@ -124,6 +124,101 @@ __device__ __forceinline__ void qs_ws(double q, double &w, double &s) {
 // x != 0 for x >= 0, on the integer pipe
 __device__ __forceinline__ bool nonzero(double x) { return __double_as_longlong(x) != 0; }
 
+// Mixed pair sums of sets without walls (LEAN): bound by instruction issue,
+// not by the FP32 pipe (pass B at 16.8M: ~165 thread instructions a pair,
+// 90 flop), so two values share an instruction where the formulas come in
+// pairs: the axes of a separation, u and v, the kernels of h_i and h_j.
+// Each half rounds like the scalar operation.
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 f2(float a, float b) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ F2 f2(float a) { return f2(a, a); }
+__device__ __forceinline__ float lo(F2 a) {
+    float x, y;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a.v));
+    return x;
+}
+__device__ __forceinline__ float hi(F2 a) {
+    float x, y;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a.v));
+    return y;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 sub2(F2 a, F2 b) { return fma2(b, f2(-1.0f), a); }
+__device__ __forceinline__ F2 clip2(F2 a) {
+    return f2(fmaxf(lo(a), 0.0f), fmaxf(hi(a), 0.0f));
+}
+__device__ __forceinline__ float frcp_ftz(float b) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(b));
+    return y;
+}
+constexpr float F32_LEAST = 1.17549435e-38f;   // least normal
+
+// The bases of the clipped quintic (qs_w above) at two q = r / h each, nh =
+// {-1 / h, -1 / h'}: one FMA a base, the product with r not rounded apart.
+struct Qs2 {
+    F2 a, b, c;
+    __device__ __forceinline__ Qs2(float r, F2 nh) {
+        const F2 rr = f2(r);
+        a = clip2(fma2(rr, nh, f2(3.0f)));
+        b = clip2(fma2(rr, nh, f2(2.0f)));
+        c = clip2(fma2(rr, nh, f2(1.0f)));
+    }
+    // s = -(dw/dq) / 5
+    __device__ __forceinline__ F2 s() const {
+        const F2 a2 = mul2(a, a), b2 = mul2(b, b), c2 = mul2(c, c);
+        return fma2(a2, a2, fma2(mul2(b2, f2(-6.0f)), b2, mul2(mul2(c2, f2(15.0f)), c2)));
+    }
+    __device__ __forceinline__ void ws(F2 &w, F2 &s) const {
+        const F2 a2 = mul2(a, a), b2 = mul2(b, b), c2 = mul2(c, c);
+        const F2 a4 = mul2(a2, a2), b4 = mul2(mul2(b2, f2(-6.0f)), b2),
+                 c4 = mul2(mul2(c2, f2(15.0f)), c2);
+        s = add2(a4, add2(b4, c4));
+        w = fma2(a4, a, fma2(b4, b, mul2(c4, c)));
+    }
+};
+
+// Separation r_i - r_j of anchor records (anchor_sep, both axes at once:
+// the same values).
+struct Sep2 {
+    F2 xi, gi, nf, invn, A;
+    __device__ __forceinline__ Sep2(const Anchor &an, const float4 &pi) {
+        const unsigned g = __float_as_uint(pi.w);
+        xi = f2(pi.x, pi.y);
+        gi = f2(anchor_gx(g), anchor_gy(g));
+        nf = f2(-an.nf[0], -an.nf[1]);
+        invn = f2(an.invn[0], an.invn[1]);
+        A = f2(an.A[0], an.A[1]);
+    }
+    __device__ __forceinline__ F2 get(const float4 &pj) const {
+        const unsigned g = __float_as_uint(pj.w);
+        F2 k = sub2(gi, f2(anchor_gx(g), anchor_gy(g)));
+        const F2 t = add2(fma2(k, invn, f2(RINT_MAGIC)), f2(-RINT_MAGIC));
+        k = fma2(t, nf, k);
+        return fma2(k, A, sub2(xi, f2(pj.x, pj.y)));
+    }
+};
+
 // Four values of one neighbour, loaded together.
 template <typename R> struct V4;
 template <> struct V4<float> { using T = float4; };

@@ -440,27 +440,39 @@ __device__ __forceinline__ bool pred_fp64(const Domain &d, double xi,
 struct Anchor {
     float A[2];      // anchor cell side per axis (float)
     float iA[2];     // 1 / side, rounded to float
+    float nf[2];     // anchor cells of a periodic axis, 0 otherwise
+    float invn[2];   // 1 / nf rounded down, 0 otherwise
     int n[2];        // anchor cells per axis
     int periodic[2];
 };
 
+// The anchor indices of a record as floats 2^23 + g (one byte permute each;
+// their differences are exact).
+__device__ __forceinline__ float anchor_gx(unsigned g) {
+    return __uint_as_float(__byte_perm(g, 0x4b000000u, 0x7410));
+}
+__device__ __forceinline__ float anchor_gy(unsigned g) {
+    return __uint_as_float(__byte_perm(g, 0x4b000000u, 0x7432));
+}
+constexpr float RINT_MAGIC = 12582912.0f;   // 1.5 2^23: t + magic - magic = rint(t)
+
 // FP32 separation r_i - r_j from anchor data: p = {xl, yl, h, gx|gy<<16}.
+// The index difference k of a periodic axis goes to its nearest image: with
+// 1 / n rounded down, |k| n^-1 passes 1/2 only where 2 |k| > n (n < 2^16),
+// so k - n rint(k / n) is exactly the wrapped index, in three operations
+// without conversions or branches; every value up to the last FMA is exact.
 __device__ __forceinline__ void anchor_sep(const Anchor &an, const float4 &pi,
                                            const float4 &pj, float &dx,
                                            float &dy) {
     const unsigned gi = __float_as_uint(pi.w), gj = __float_as_uint(pj.w);
-    int kx = (int)(gi & 0xffffu) - (int)(gj & 0xffffu);
-    int ky = (int)(gi >> 16) - (int)(gj >> 16);
-    if (an.periodic[0]) {
-        if (2 * kx > an.n[0]) kx -= an.n[0];
-        else if (2 * kx < -an.n[0]) kx += an.n[0];
-    }
-    if (an.periodic[1]) {
-        if (2 * ky > an.n[1]) ky -= an.n[1];
-        else if (2 * ky < -an.n[1]) ky += an.n[1];
-    }
-    dx = fmaf((float)kx, an.A[0], pi.x - pj.x);
-    dy = fmaf((float)ky, an.A[1], pi.y - pj.y);
+    float kx = anchor_gx(gi) - anchor_gx(gj);
+    float ky = anchor_gy(gi) - anchor_gy(gj);
+    const float tx = __fadd_rn(__fmaf_rn(kx, an.invn[0], RINT_MAGIC), -RINT_MAGIC);
+    const float ty = __fadd_rn(__fmaf_rn(ky, an.invn[1], RINT_MAGIC), -RINT_MAGIC);
+    kx = __fmaf_rn(-tx, an.nf[0], kx);
+    ky = __fmaf_rn(-ty, an.nf[1], ky);
+    dx = fmaf(kx, an.A[0], pi.x - pj.x);
+    dy = fmaf(ky, an.A[1], pi.y - pj.y);
 }
 
 // Anchor record {xl, yl, h, gx | gy << 16} of a position: anchor cell g =
@@ -494,8 +506,8 @@ __device__ __forceinline__ float4 anchor_record(double x, double y, float h,
 // data p = {xl, yl, h, gx | gy << 16}.
 __device__ __forceinline__ float2 anchor_rel(const Anchor &an, const float4 &p) {
     const unsigned g = __float_as_uint(p.w);
-    return make_float2(fmaf((float)(g & 0xffffu), an.A[0], p.x),
-                       fmaf((float)(g >> 16), an.A[1], p.y));
+    return make_float2(fmaf(anchor_gx(g) - 8388608.0f, an.A[0], p.x),
+                       fmaf(anchor_gy(g) - 8388608.0f, an.A[1], p.y));
 }
 
 // Membership of a candidate whose FP32 anchor separation r2 is already

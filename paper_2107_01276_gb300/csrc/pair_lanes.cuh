@@ -46,7 +46,7 @@ __device__ __forceinline__ bool skin_member(const Domain &d, const Anchor &an,
 // against the kernel at its inflection point for h_ij = (h_i + h_j)/2),
 // limited to 0.25 h_i (Eq. shift-limit).  finish() also writes the two
 // per-particle records pass B gathers: {m, V = m/rho, rho, 1/(rho^2 beta)}
-// and {p, u, v, 1/h}.
+// and {u, v, p, 1/h}.
 template <typename R, bool LEAN>
 struct PassALane {
     static constexpr bool L64 = lean64<R, LEAN>;
@@ -107,6 +107,26 @@ struct PassALane {
         }
     }
 
+    // mixed, LEAN: every kernel term of an entry that is no member (in
+    // false) is zero by its clip; constants are applied in finish()
+    __device__ __forceinline__ void pair2(R mj, R hj, R pj, bool in, F2 d, R r2,
+                                          F2 &acc) {
+        const R rinv = frsqrt(fmaxf(r2, F32_LEAST));
+        const R r = r2 * rinv;
+        const R hsinv = frcp_ftz(hi + hj);
+        F2 w, s;
+        Qs2(r, f2(-hinv, R(-2) * hsinv)).ws(w, s);
+        rho = fmaf(mj, lo(w), rho);
+        srw = fmaf(mj * r, lo(s), srw);
+        psum += in ? pj : R(0);
+        cnt += in ? 1 : 0;
+        R ratio = sph::hi(w) * inv_wxi;
+        ratio *= ratio;
+        const R f = mj * fmaf(R(0.24) * ratio, ratio, R(1)) *
+                    (hsinv * hsinv * hsinv) * (sph::hi(s) * rinv);
+        acc = fma2(f2(f), d, acc);
+    }
+
     // wall neighbours of particle i (section 2.2): mass m_w in rho, beta
     // and the shift, p_w in p_avg
     template <int T>
@@ -131,7 +151,7 @@ struct PassALane {
         ay = team_sum<T>(tm.mask, ay);
         cnt = team_sum<T>(tm.mask, cnt);
         if (tm.lane != 0) return;
-        if constexpr (L64) {
+        if constexpr (LEAN) {
             srw *= R(-5);
             ax *= R(-40) * sigma_norm<R>();
             ay *= R(-40) * sigma_norm<R>();
@@ -169,7 +189,7 @@ struct PassALane {
         a.rb2[i] = rb2;
         typename V4<R>::T A, B;
         A.x = mi; A.y = V; A.z = rho; A.w = rb2;
-        B.x = a.p[i]; B.y = a.u[i]; B.z = a.v[i]; B.w = hinv;
+        B.x = a.u[i]; B.y = a.v[i]; B.z = a.p[i]; B.w = hinv;
         a.nbA[i] = A;
         a.nbB[i] = B;
     }
@@ -212,9 +232,9 @@ struct PassBLane {
         hinv = Bi.w;
         dsig_i = L64 ? hinv * hinv * hinv : sigma_norm<R>() * hinv * hinv * hinv;
         rho_i = a.rho[i];
-        pi = Bi.x;
-        ui = Bi.y;
-        vi = Bi.z;
+        ui = Bi.x;
+        vi = Bi.y;
+        pi = Bi.z;
         pavg_i = a.pavg[i];
         Pi = (pi - pavg_i) * rb2i;
         const R hi = R(1) / hinv;
@@ -281,14 +301,48 @@ struct PassBLane {
         vy += visc * (vi - ugy);
     }
 
+    // mixed, LEAN: the same sums less constant factors, which finish()
+    // applies (-5 sigma of both gradients, 1/2 of their mean, the force's
+    // sign); sums = {div, diff}, force and viscous vectors
+    struct Sums2 {
+        F2 f, w;
+    };
+    __device__ __forceinline__ void pair2(F2 d, const float4 &A, const float4 &B, R pref,
+                                          F2 uvi, R hi3, Sums2 &S) {
+        const R r2 = fmaf(lo(d), lo(d), hi(d) * hi(d));
+        const R rinv = frsqrt(fmaxf(r2, F32_LEAST));
+        const F2 g = mul2(mul2(Qs2(r2 * rinv, f2(-hinv, -B.w)).s(), f2(rinv)),
+                          f2(hi3, B.w * B.w * B.w));
+        const R gi = lo(g), gj = hi(g);
+        const R inv_reta = frcp_ftz(r2 + eta);
+        const R rdg = (gi + gj) * r2;
+        const R rdge = rdg * inv_reta;
+        const F2 uv = sub2(uvi, f2(B.x, B.y));
+        const F2 ud = mul2(uv, d);
+        div = fmaf(A.y * gi, lo(ud) + hi(ud), div);
+        diff = fmaf(A.y * frcp_ftz(hinv + B.w) * (dden_on ? rdge : rdg), pi - B.z, diff);
+        const R mfp = A.x * fmaf(Pi, gi, (B.z - pref) * A.w * gj);
+        S.f = fma2(f2(mfp), d, S.f);
+        S.w = fma2(f2(A.x * rdge * frcp_ftz(rho_i + A.z)), uv, S.w);
+    }
+    __device__ __forceinline__ void take(const Sums2 &S) {
+        const R k = R(-5) * sigma_norm<R>();
+        div *= k;
+        diff *= R(0.5) * k;
+        fax = -k * lo(S.f);
+        fay = -k * hi(S.f);
+        vx = R(0.5) * k * lo(S.w);
+        vy = R(0.5) * k * hi(S.w);
+    }
+
     // list neighbour j with its pass-B records A = {m, V, rho, 1/(rho^2
-    // beta)}, B = {p, u, v, 1/h}; pref: p_avg,i, or p_avg,j (literal
+    // beta)}, B = {u, v, p, 1/h}; pref: p_avg,i, or p_avg,j (literal
     // reading, pavg_mode 1)
     template <typename V>
     __device__ __forceinline__ void pair_rec(R dx, R dy, R r2, const V &A,
                                              const V &B, R pref) {
-        pair(dx, dy, r2, B.w, A.x, A.y, A.z, (B.x - pref) * A.w, B.x, B.y,
-             B.z, B.y, B.z);
+        pair(dx, dy, r2, B.w, A.x, A.y, A.z, (B.z - pref) * A.w, B.z, B.x,
+             B.y, B.x, B.y);
     }
 
     template <int T>
@@ -362,7 +416,18 @@ __device__ __forceinline__ void pass_a_list(const PassAArgs<R> &a, int i,
     if constexpr (sizeof(R) == 4) {
         // U list entries per step, their records loaded before any is used
         // (more loads in flight per warp)
+        [[maybe_unused]] const Sep2 sp2(a.an, sp.pi);
+        [[maybe_unused]] F2 acc = f2(0.0f);
         auto body = [&](int j, const float4 &pj, R mj, R pjv) {
+            if constexpr (LEAN) {
+                // r = 0 (i itself): the gradient sums add zero by s = 0, d = 0
+                const F2 d = sp2.get(pj);
+                const R r2 = fmaf(lo(d), lo(d), sph::hi(d) * sph::hi(d));
+                const bool in = !a.filter || skin_member<R>(a.d, a.an, r2, hi, pj.z, xid,
+                                                            yid, hid, a.x, a.y, a.h, j);
+                L.pair2(mj, pj.z, pjv, in, d, r2, acc);
+                return;
+            }
             R dx, dy;
             anchor_sep(a.an, sp.pi, pj, dx, dy);
             const R r2 = fmaf(dx, dx, dy * dy);
@@ -397,6 +462,10 @@ __device__ __forceinline__ void pass_a_list(const PassAArgs<R> &a, int i,
             if (!SPH_DCHECK((unsigned)j < (unsigned)a.n)) j = i;
             body(j, __ldg(&a.pk[j]), a.m[j], a.p[j]);
         }
+        if constexpr (LEAN) {
+            L.ax = lo(acc);
+            L.ay = sph::hi(acc);
+        }
     } else {
         for (uint32_t k = b + tm.lane; k < e; k += T) {
             const int j = (int)__ldg(&a.list[k]);
@@ -425,8 +494,16 @@ __device__ __forceinline__ void pass_b_list(const PassBArgs<R> &a, int i,
     if constexpr (sizeof(R) == 4) {
         // neither a membership test for skin entries nor a test for i
         // itself: both add exactly zero
+        [[maybe_unused]] const Sep2 sp2(a.an, sp.pi);
+        [[maybe_unused]] const F2 uvi = f2(L.ui, L.vi);
+        [[maybe_unused]] const R hi3 = L.hinv * L.hinv * L.hinv;
+        [[maybe_unused]] typename PassBLane<R, LEAN>::Sums2 S{f2(0.0f), f2(0.0f)};
         auto body = [&](int j, const float4 &pj, const float4 &A,
                         const float4 &B) {
+            if constexpr (LEAN) {
+                L.pair2(sp2.get(pj), A, B, literal ? a.pavg[j] : pavg_i, uvi, hi3, S);
+                return;
+            }
             R dx, dy;
             anchor_sep(a.an, sp.pi, pj, dx, dy);
             L.pair_rec(dx, dy, fmaf(dx, dx, dy * dy), A, B,
@@ -456,6 +533,7 @@ __device__ __forceinline__ void pass_b_list(const PassBArgs<R> &a, int i,
             if (!SPH_DCHECK((unsigned)j < (unsigned)a.n)) j = i;
             body(j, __ldg(&a.pk[j]), a.nbA[j], a.nbB[j]);
         }
+        if constexpr (LEAN) L.take(S);
     } else {
         for (uint32_t k = b + tm.lane; k < e; k += T) {
             const int j = (int)__ldg(&a.list[k]);

@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(BATCH_THREADS)
         const PassAArgs<R> &a = args[q];
         const int i = (item - __ldg(&sp.first[q])) * batch_rows(T) + (int)threadIdx.x / T;
         if (i >= a.n) continue;
-        if (sizeof(R) == 4 || a.w.n > 0)
+        if (a.w.n > 0)
             pass_a_at<R, T, true>(a, i, tm);
         else
             pass_a_at<R, T, false>(a, i, tm);
@@ -462,7 +462,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, sizeof(R) == 4 ? 5 : 1)
         const PassBArgs<R> &a = args[q];
         const int i = (item - __ldg(&sp.first[q])) * batch_rows(T) + (int)threadIdx.x / T;
         if (i >= a.n) continue;
-        if (sizeof(R) == 4 || a.w.n > 0)
+        if (a.w.n > 0)
             pass_b_at<R, T, true>(a, i, tm);
         else
             pass_b_at<R, T, false>(a, i, tm);
