@@ -328,11 +328,49 @@ __global__ void __launch_bounds__(128) k_list_fill_queue(ListArgs a) {
 constexpr int TILE_CAP = 256;   // staged candidates per warp and batch
 constexpr int TILE_LD = 2;      // candidate loads in flight per lane
 
+// The grid's levels in shared memory, a lane per level in the walk's set-up.
+struct LevTab {
+    float cf[MAX_LEVELS], invw[2][MAX_LEVELS], w[2][MAX_LEVELS], invP[2][MAX_LEVELS];
+    int n[2][MAX_LEVELS], bb[4][MAX_LEVELS];
+    // the whole block; ends with a barrier
+    __device__ __forceinline__ void load(const Grid &g) {
+        const int l = threadIdx.x;
+        if (l < MAX_LEVELS) {
+            const Level &L = g.lev[l];
+            cf[l] = L.cf;
+#pragma unroll
+            for (int ax = 0; ax < 2; ++ax) {
+                invw[ax][l] = L.invw[ax];
+                w[ax][l] = L.wf[ax];
+                invP[ax][l] = L.invP[ax];
+                n[ax][l] = L.n[ax];
+            }
+#pragma unroll
+            for (int t = 0; t < 4; ++t) bb[t][l] = __ldg(&g.bbox[4 * l + t]);
+        }
+        __syncthreads();
+    }
+};
+constexpr int TILE_LEV = 16;    // levels set up at once, a lane each
+// first cell and cell count of the three pieces of each axis, per level
+constexpr int TILE_PCS = 12 * TILE_LEV;
+
+__device__ __forceinline__ float warp_min(float v) {
+    float r;
+    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float warp_max(float v) {
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+
 // Squared gap between the box [xc - hx, xc + hx] x [yc - hy, yc + hy] and
-// cell (cx, cy) of level L (unwrapped indices), less a margin far above
+// cell (cx, cy) of level l (unwrapped indices), less a margin far above
 // FP32 rounding; periodic axes use the nearest image of the cell, the edge
 // cells of a non-periodic axis reach to infinity.
-__device__ __forceinline__ float box_gap2(const Domain &d, const Level &L,
+__device__ __forceinline__ float box_gap2(const Domain &d, const LevTab &T, int l,
                                           int cx, int cy, float xc, float yc,
                                           float hx, float hy) {
     const int c[2] = {cx, cy};
@@ -340,18 +378,18 @@ __device__ __forceinline__ float box_gap2(const Domain &d, const Level &L,
     float g2 = 0.0f;
 #pragma unroll
     for (int ax = 0; ax < 2; ++ax) {
-        const float w = L.wf[ax];
+        const float w = T.w[ax][l];
         const float m = 1e-5f * (fabsf(q[ax]) + hh[ax] + w);
         float gap;
         if (d.periodic[ax]) {
-            const float P = (float)L.n[ax] * w;
+            const float P = (float)T.n[ax][l] * w;
             float t = q[ax] - ((float)c[ax] + 0.5f) * w;
-            t -= P * rintf(t * L.invP[ax]);
+            t -= P * rintf(t * T.invP[ax][l]);
             gap = fabsf(t) - 0.5f * w - hh[ax];
         } else {
             float lo = (float)c[ax] * w, hi = lo + w;
             if (c[ax] <= 0) lo = -3.0e38f;
-            if (c[ax] >= L.n[ax] - 1) hi = 3.0e38f;
+            if (c[ax] >= T.n[ax][l] - 1) hi = 3.0e38f;
             gap = fmaxf(lo - (q[ax] + hh[ax]), (q[ax] - hh[ax]) - hi);
         }
         gap = fmaxf(0.0f, gap - m);
@@ -377,8 +415,8 @@ __device__ __forceinline__ float box_gap2(const Domain &d, const Level &L,
 // records its chunk's reference and span, so that pass takes the same
 // decisions with the same arithmetic.
 template <bool DIRECT, int T>
-__device__ __forceinline__ void tile_chunk(const ListArgs &a, float4 *sc,
-                                           int *pcs, int lc, uint32_t cs,
+__device__ __forceinline__ void tile_chunk(const ListArgs &a, const LevTab &tab,
+                                           float4 *sc, int *pcs, int lc, uint32_t cs,
                                            uint32_t pe, uint32_t p0, int only,
                                            int span = 1) {
     static_assert(T == 1 || T == 4 || T == 16, "team of 1, 4 or 16 lanes");
@@ -387,99 +425,119 @@ __device__ __forceinline__ void tile_chunk(const ListArgs &a, float4 *sc,
     const uint32_t i = p0 + (uint32_t)(lane / T);
     const bool act = i < pe && (only < 0 || (int)i == only);
     const float4 pC = __ldg(&a.pk[cs]);
-    float rxi = 0.0f, ryi = 0.0f, Ri = 0.0f;
-    float xlo = 3.0e38f, xhi = -3.0e38f, ylo = 3.0e38f, yhi = -3.0e38f, hmx = 0.0f;
+    float rxi = 0.0f, ryi = 0.0f, Ri = 0.0f, hmx = 0.0f;
     // the chunk's bounding box in reference-relative coordinates
     float rxlo = 3.0e38f, rxhi = -3.0e38f, rylo = 3.0e38f, ryhi = -3.0e38f;
     if (act) {
         const float4 pi = __ldg(&a.pk[i]);
         anchor_sep(a.an, pi, pC, rxi, ryi);
         Ri = a.skin * (3.0f * pi.z);
-        const float2 q = anchor_rel(a.an, pi);
-        xlo = xhi = q.x;
-        ylo = yhi = q.y;
         hmx = pi.z;
         rxlo = rxhi = rxi;
         rylo = ryhi = ryi;
     }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        xlo = fminf(xlo, __shfl_xor_sync(0xffffffffu, xlo, o));
-        xhi = fmaxf(xhi, __shfl_xor_sync(0xffffffffu, xhi, o));
-        ylo = fminf(ylo, __shfl_xor_sync(0xffffffffu, ylo, o));
-        yhi = fmaxf(yhi, __shfl_xor_sync(0xffffffffu, yhi, o));
-        hmx = fmaxf(hmx, __shfl_xor_sync(0xffffffffu, hmx, o));
-        rxlo = fminf(rxlo, __shfl_xor_sync(0xffffffffu, rxlo, o));
-        rxhi = fmaxf(rxhi, __shfl_xor_sync(0xffffffffu, rxhi, o));
-        rylo = fminf(rylo, __shfl_xor_sync(0xffffffffu, rylo, o));
-        ryhi = fmaxf(ryhi, __shfl_xor_sync(0xffffffffu, ryhi, o));
-    }
-    const float xc = 0.5f * (xlo + xhi), yc = 0.5f * (ylo + yhi);
-    const float bx = 0.5f * (xhi - xlo), by = 0.5f * (yhi - ylo);
+    rxlo = warp_min(rxlo);
+    rxhi = warp_max(rxhi);
+    rylo = warp_min(rylo);
+    ryhi = warp_max(ryhi);
+    hmx = warp_max(hmx);
+    // the same box from the domain's corner (a chunk does not straddle a
+    // period); its rounding is far below the margins of the cell ranges
+    const float2 qC = anchor_rel(a.an, pC);
+    const float xc = qC.x + 0.5f * (rxlo + rxhi), yc = qC.y + 0.5f * (rylo + ryhi);
+    const float bx = 0.5f * (rxhi - rxlo), by = 0.5f * (ryhi - rylo);
     const float Rmx = a.skin * (3.0f * hmx);   // largest pair radius of a chunk particle
     const uint32_t W = a.stage_w;
     uint32_t k = 0;
     if (DIRECT && act) k = a.off[i];
     uint32_t *row = a.stage + (size_t)i * W;
-    const Level &LC = a.g.lev[lc];
     const float Amax = fmaxf(a.an.A[0], a.an.A[1]);
     const float Lx = (float)a.d.L[0], Ly = (float)a.d.L[1];
     const float iLx = 1.0f / Lx, iLy = 1.0f / Ly;
     const bool exact = !(a.skin > 1.0f);
-    const uint32_t lmask = a.g.level_mask & ~((1u << lc) - 1u);
-    for (uint32_t mm = lmask; mm; mm &= mm - 1) {
-        const int l = __ffs(mm) - 1;
-        const int *bb = a.g.bbox + 4 * l;
-        if (__ldg(&bb[0]) > __ldg(&bb[1])) continue;   // level holds no particle
-        const Level &L = a.g.lev[l];
-        const float Rl = a.skin * fmaxf(3.0f * hmx, L.cf);
-        const float Q = Rl * (1.0f + 1e-5f);
-        AxisPieces px, py;
-        if (!axis_pieces(a.d, L, bb, 0, xc, bx + Q, px)) continue;
-        if (!axis_pieces(a.d, L, bb, 1, yc, by + Q, py)) continue;
-        // per-level constants (functions of lc and l only)
-        const float reach = a.skin * L.cf + (float)span * fmaxf(LC.wf[0], LC.wf[1]) +
-                            fmaxf(L.wf[0], L.wf[1]);
-        const bool wrapx = a.d.periodic[0] && 2.0f * (reach + 4.0f * a.an.A[0]) >= Lx;
-        const bool wrapy = a.d.periodic[1] && 2.0f * (reach + 4.0f * a.an.A[1]) >= Ly;
-        const bool wrap = wrapx || wrapy;
-        const float G = reach + (wrap ? fmaxf(Lx, Ly) : 0.0f);
-        const float KB = 4.0f * Amax + G;
-        const bool coarse = l > lc;
-        // the query's cell pieces go to shared memory: nothing of them stays
-        // in registers through the staging and test loops
+    uint32_t mm = a.g.level_mask & ~((1u << lc) - 1u);
+    while (mm) {
+        // set-up of up to TILE_LEV levels, lane t: level lb + t
+        const int lb = __ffs(mm) - 1;
+        const int lt = lb + lane;
+        int nc = 0;
+        bool wx = false, wy = false;
+        float KB = 0.0f;
         __syncwarp();
-        if (lane == 0) {
+        if (lane < TILE_LEV && lt < MAX_LEVELS && ((mm >> lt) & 1u) &&
+            tab.bb[0][lt] <= tab.bb[1][lt]) {
+            const float Q = a.skin * fmaxf(3.0f * hmx, tab.cf[lt]) * (1.0f + 1e-5f);
+            AxisPieces px, py;
+            if (axis_pieces_of(a.d.periodic[0], tab.n[0][lt], tab.invw[0][lt], tab.bb[0][lt],
+                               tab.bb[1][lt], xc, bx + Q, px) &&
+                axis_pieces_of(a.d.periodic[1], tab.n[1][lt], tab.invw[1][lt], tab.bb[2][lt],
+                               tab.bb[3][lt], yc, by + Q, py)) {
+                int nx = 0, ny = 0;
 #pragma unroll
-            for (int t = 0; t < 3; ++t) {
-                pcs[t] = px.first[t];
-                pcs[3 + t] = px.shift[t];
-                pcs[6 + t] = max(0, px.last[t] - px.first[t] + 1);
-                pcs[9 + t] = py.first[t];
-                pcs[12 + t] = py.shift[t];
-                pcs[15 + t] = max(0, py.last[t] - py.first[t] + 1);
+                for (int t = 0; t < 3; ++t) {
+                    const int cx = max(0, px.last[t] - px.first[t] + 1);
+                    const int cy = max(0, py.last[t] - py.first[t] + 1);
+                    pcs[t * TILE_LEV + lane] = px.first[t];
+                    pcs[(3 + t) * TILE_LEV + lane] = cx;
+                    pcs[(6 + t) * TILE_LEV + lane] = py.first[t];
+                    pcs[(9 + t) * TILE_LEV + lane] = cy;
+                    nx += cx;
+                    ny += cy;
+                }
+                nc = nx * ny;
+                const float reach = a.skin * tab.cf[lt] +
+                                    (float)span * fmaxf(tab.w[0][lc], tab.w[1][lc]) +
+                                    fmaxf(tab.w[0][lt], tab.w[1][lt]);
+                wx = a.d.periodic[0] && 2.0f * (reach + 4.0f * a.an.A[0]) >= Lx;
+                wy = a.d.periodic[1] && 2.0f * (reach + 4.0f * a.an.A[1]) >= Ly;
+                KB = 4.0f * Amax + reach + (wx || wy ? fmaxf(Lx, Ly) : 0.0f);
             }
         }
+        mm = lb + TILE_LEV < MAX_LEVELS ? mm & ~((1u << (lb + TILE_LEV)) - 1u) : 0u;
+        int ninc = nc;
+#pragma unroll
+        for (int o = 1; o < TILE_LEV; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, ninc, o);
+            if (lane >= o) ninc += t;
+        }
+        const int ncell = __shfl_sync(0xffffffffu, ninc, TILE_LEV - 1);
+        if (ncell == 0) continue;
+        const bool wrapx = __any_sync(0xffffffffu, wx);
+        const bool wrapy = __any_sync(0xffffffffu, wy);
+        const bool wrap = wrapx || wrapy;
+        KB = warp_max(KB);
         __syncwarp();
-        const int nx = pcs[6] + pcs[7] + pcs[8];
-        const int ncell = nx * (pcs[15] + pcs[16] + pcs[17]);
-        const uint64_t lbits = (uint64_t)l << (2 * a.g.mbits);
         for (int base = 0; base < ncell; base += 32) {
-            // lane -> one cell of the query (row-major, unwrapped order)
-            uint32_t s = 0, e = 0;
-            const int idx = base + lane;
+            // lane -> one cell of the query (level by level, row-major,
+            // unwrapped order)
+            uint32_t s = 0, e = 0, co = 0;
+            const int idx = base + lane, idc = min(idx, ncell - 1);
+            int sl = 0;
+#pragma unroll
+            for (int st = TILE_LEV / 2; st; st >>= 1) {
+                const int v = __shfl_sync(0xffffffffu, ninc, sl + st - 1);
+                if (v <= idc) sl += st;
+            }
+            const int loc = idc - __shfl_sync(0xffffffffu, ninc - nc, sl);
             if (idx < ncell) {
-                const int iy = idx / nx;
-                int ix = idx - iy * nx, jy = iy;
+                const int l = lb + sl;
+                const int *pc = pcs + sl;
+                const int nx0 = pc[3 * TILE_LEV], nx1 = pc[4 * TILE_LEV];
+                const int ny0 = pc[9 * TILE_LEV], ny1 = pc[10 * TILE_LEV];
+                const int nx = nx0 + nx1 + pc[5 * TILE_LEV];
+                int jy = loc / nx, ix = loc - jy * nx;
                 int kx = 0, ky = 0;
-                while (kx < 2 && ix >= pcs[6 + kx]) ix -= pcs[6 + kx++];
-                while (ky < 2 && jy >= pcs[15 + ky]) jy -= pcs[15 + ky++];
-                const int cx = pcs[kx] + ix, sx = pcs[3 + kx];
-                const int cy = pcs[9 + ky] + jy, sy = pcs[12 + ky];
-                const float g2 = box_gap2(a.d, L, cx, cy, xc, yc, bx, by);
+                if (ix >= nx0) { ix -= nx0; kx = 1; if (ix >= nx1) { ix -= nx1; kx = 2; } }
+                if (jy >= ny0) { jy -= ny0; ky = 1; if (jy >= ny1) { jy -= ny1; ky = 2; } }
+                const int cx = pc[kx * TILE_LEV] + ix, cy = pc[(6 + ky) * TILE_LEV] + jy;
+                // pieces 0 and 2 lie a period off (periodic axes only)
+                const int sx = (1 - kx) * tab.n[0][l], sy = (1 - ky) * tab.n[1][l];
+                const float Rl = a.skin * fmaxf(3.0f * hmx, tab.cf[l]);
+                const float g2 = box_gap2(a.d, tab, l, cx, cy, xc, yc, bx, by);
                 float hc;
                 if (g2 < Rl * Rl &&
-                    table_lookup(a.g, lbits | (spread2((uint64_t)(cy + sy)) << 1) |
+                    table_lookup(a.g, ((uint64_t)l << (2 * a.g.mbits)) |
+                                          (spread2((uint64_t)(cy + sy)) << 1) |
                                           spread2((uint64_t)(cx + sx)),
                                  s, e, &hc)) {
                     const float Rc = a.skin * 3.0f * fmaxf(hmx, hc);
@@ -488,6 +546,7 @@ __device__ __forceinline__ void tile_chunk(const ListArgs &a, float4 *sc,
                 } else {
                     s = e = 0;
                 }
+                co = l > lc ? STAGE_COARSE : 0u;
             }
             const uint32_t cnt = e - s;
             uint32_t inc = cnt;
@@ -498,6 +557,7 @@ __device__ __forceinline__ void tile_chunk(const ListArgs &a, float4 *sc,
             }
             const uint32_t total = __shfl_sync(0xffffffffu, inc, 31);
             const uint32_t exc = inc - cnt;
+            s |= co;   // staged indices carry it
             for (uint32_t q0 = 0; q0 < total; q0 += TILE_CAP) {
                 const uint32_t mq = min((uint32_t)TILE_CAP, total - q0);
                 // stage: candidate q0 + u; its cell is the first lane whose
@@ -509,7 +569,9 @@ __device__ __forceinline__ void tile_chunk(const ListArgs &a, float4 *sc,
                 // not staged; the others keep their order (ballot
                 // compaction), so the test loop sees the same members in the
                 // same order.
-                uint32_t m = 0;
+                // m: staged; mf: of them on the chunk's own level (they come
+                // first)
+                uint32_t m = 0, mf = 0;
                 for (uint32_t u0 = 0; u0 < mq; u0 += 32 * TILE_LD) {
                     float4 v[TILE_LD];
                     uint32_t jj[TILE_LD];
@@ -526,7 +588,7 @@ __device__ __forceinline__ void tile_chunk(const ListArgs &a, float4 *sc,
                         const uint32_t st0 = __shfl_sync(0xffffffffu, s, pos);
                         const uint32_t ex0 = __shfl_sync(0xffffffffu, exc, pos);
                         jj[r] = st0 + (qq - ex0);
-                        if (u < mq) v[r] = __ldg(&a.pk[jj[r]]);
+                        if (u < mq) v[r] = __ldg(&a.pk[jj[r] & ~STAGE_COARSE]);
                     }
 #pragma unroll
                     for (int r = 0; r < TILE_LD; ++r) {
@@ -549,20 +611,23 @@ __device__ __forceinline__ void tile_chunk(const ListArgs &a, float4 *sc,
                             sc[m + (uint32_t)__popc(kb & ((1u << lane) - 1u))] =
                                 make_float4(rx, ry, Rj, __uint_as_float(jj[r]));
                         m += (uint32_t)__popc(kb);
+                        mf += (uint32_t)__popc(
+                            kb & __ballot_sync(0xffffffffu, !(jj[r] & STAGE_COARSE)));
                     }
                 }
                 __syncwarp();
                 {
-                    // one loop per (exact, wrap, coarse) case, branch-free in
-                    // the common ones: a predicated store and a counter.  A
-                    // team of T lanes takes T consecutive candidates per
-                    // iteration; the ballot keeps the team's entries in
-                    // candidate order.
-                    auto test = [&](auto ex_c, auto wr_c, auto co_c) {
+                    // one loop per (exact, wrap) case and own / coarser
+                    // level, branch-free in the common ones: a predicated
+                    // store and a counter.  A team of T lanes takes T
+                    // consecutive candidates per iteration; the ballot keeps
+                    // the team's entries in candidate order.
+                    auto test = [&](auto ex_c, auto wr_c, auto co_c, uint32_t ub, uint32_t ue) {
                         constexpr bool EX = decltype(ex_c)::value;
                         constexpr bool WR = decltype(wr_c)::value;
                         constexpr bool CO = decltype(co_c)::value;
-                        auto pair_in = [&](uint32_t u, uint32_t &j) {
+                        // ent: the candidate's index, with STAGE_COARSE if CO
+                        auto pair_in = [&](uint32_t u, uint32_t &ent) {
                             const float4 c = sc[u];
                             float dx = rxi - c.x, dy = ryi - c.y;
                             if (WR) {
@@ -572,19 +637,22 @@ __device__ __forceinline__ void tile_chunk(const ListArgs &a, float4 *sc,
                             const float r2 = fmaf(dx, dx, dy * dy);
                             const float R = fmaxf(Ri, c.z);
                             const float R2 = R * R;
-                            j = __float_as_uint(c.w);
+                            ent = __float_as_uint(c.w);
                             bool in = r2 < R2;
                             if (EX) {
                                 const float band = fmaf(R, KB, R2) * (1.0f / 65536.0f);
                                 in = r2 < R2 - band;
-                                if (!in && !(r2 > R2 + band))
+                                if (!in && !(r2 > R2 + band)) {
+                                    const uint32_t j = CO ? ent & ~STAGE_COARSE : ent;
                                     in = pred_fp64(a.d, __ldg(&a.x[i]), __ldg(&a.y[i]),
                                                    __ldg(&a.h[i]), __ldg(&a.x[j]),
                                                    __ldg(&a.y[j]), __ldg(&a.h[j]));
+                                }
                             }
                             return in;
                         };
-                        auto put = [&](uint32_t pos, uint32_t j) {
+                        auto put = [&](uint32_t pos, uint32_t ent) {
+                            const uint32_t j = CO ? ent & ~STAGE_COARSE : ent;
                             if (DIRECT) {
                                 if (pos < a.cap) a.list[pos] = j;
                                 if (CO) {
@@ -593,52 +661,48 @@ __device__ __forceinline__ void tile_chunk(const ListArgs &a, float4 *sc,
                                     if (rp < a.cap) a.list[rp] = i;
                                 }
                             } else {
-                                if (pos < W) row[pos] = CO ? (j | STAGE_COARSE) : j;
+                                if (pos < W) row[pos] = ent;
                                 if (CO) atomicAdd(&a.rev[j], 1u);
                             }
                         };
                         if constexpr (T == 1) {
                             if (!act) return;
 #pragma unroll 4
-                            for (uint32_t u = 0; u < m; ++u) {
-                                uint32_t j;
-                                const bool in = pair_in(u, j);
+                            for (uint32_t u = ub; u < ue; ++u) {
+                                uint32_t ent;
+                                const bool in = pair_in(u, ent);
                                 if (DIRECT) {
-                                    if (in) put(k, j);
+                                    if (in) put(k, ent);
                                 } else {
-                                    if (in && k < W) row[k] = CO ? (j | STAGE_COARSE) : j;
-                                    if (CO && in) atomicAdd(&a.rev[j], 1u);
+                                    if (in && k < W) row[k] = ent;
+                                    if (CO && in) atomicAdd(&a.rev[ent & ~STAGE_COARSE], 1u);
                                 }
                                 k += in ? 1u : 0u;
                             }
                         } else {
                             const unsigned gsh = (unsigned)(lane & ~(T - 1));
                             const unsigned below = (1u << sub) - 1u;
-                            for (uint32_t u0 = 0; u0 < m; u0 += T) {
+                            for (uint32_t u0 = ub; u0 < ue; u0 += T) {
                                 const uint32_t u = u0 + (uint32_t)sub;
-                                uint32_t j = 0;
-                                const bool in = act && u < m && pair_in(u, j);
+                                uint32_t ent = 0;
+                                const bool in = act && u < ue && pair_in(u, ent);
                                 const unsigned gb = (__ballot_sync(0xffffffffu, in) >> gsh) &
                                                     ((1u << T) - 1u);
-                                if (in) put(k + (uint32_t)__popc(gb & below), j);
+                                if (in) put(k + (uint32_t)__popc(gb & below), ent);
                                 k += (uint32_t)__popc(gb);
                             }
                         }
                     };
                     using TT = std::true_type;
                     using FF = std::false_type;
+                    auto both = [&](auto ex, auto wr) {
+                        test(ex, wr, FF(), 0u, mf);
+                        if (mf < m) test(ex, wr, TT(), mf, m);
+                    };
                     if (exact) {
-                        if (wrap) {
-                            if (coarse) test(TT(), TT(), TT()); else test(TT(), TT(), FF());
-                        } else {
-                            if (coarse) test(TT(), FF(), TT()); else test(TT(), FF(), FF());
-                        }
+                        if (wrap) both(TT(), TT()); else both(TT(), FF());
                     } else {
-                        if (wrap) {
-                            if (coarse) test(FF(), TT(), TT()); else test(FF(), TT(), FF());
-                        } else {
-                            if (coarse) test(FF(), FF(), TT()); else test(FF(), FF(), FF());
-                        }
+                        if (wrap) both(FF(), TT()); else both(FF(), FF());
                     }
                 }
                 __syncwarp();
@@ -677,24 +741,39 @@ template <int T, bool MERGE = false>
 __global__ void __launch_bounds__(128, MERGE ? SPH_TILE_MERGE_BLOCKS : (T == 1 ? 7 : 6))
     k_list_tile(ListArgs a) {
     __shared__ float4 sbuf[4][TILE_CAP];
-    __shared__ int spcs[4][20];
+    __shared__ int spcs[4][TILE_PCS];
+    __shared__ LevTab tab;
+    tab.load(a.g);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t gw = blockIdx.x * 4u + (uint32_t)w;
     const uint32_t n = (uint32_t)a.n;
     if constexpr (T == 1) {
         const uint32_t base = gw * 32u;
         if (base >= n) return;
+        // the keys of the range, in registers: cells end where the next
+        // begins, but for the last one, whose end the table holds
         const uint32_t i = base + lane;
-        const bool head = i < n && (i == 0 || a.skey[i] != a.skey[i - 1]);
-        unsigned heads = __ballot_sync(0xffffffffu, head);
+        const uint64_t key = i < n ? a.skey[i] : EMPTY_KEY;
+        uint64_t prev = __shfl_up_sync(0xffffffffu, key, 1);
+        if (lane == 0 && i > 0) prev = a.skey[i - 1];
+        const bool head = i < n && (i == 0 || prev != key);
+        const unsigned all = __ballot_sync(0xffffffffu, head);
+        unsigned heads = all;
+        if (!heads) return;
+        uint32_t ls, le = n;
+        table_lookup(a.g, __shfl_sync(0xffffffffu, key, 31 - __clz(all)), ls, le);
+        auto cell_end = [&](uint32_t h) {   // h: lane of the cell's first particle
+            const unsigned up = all & ~((2u << h) - 1u);
+            return up ? base + (uint32_t)(__ffs(up) - 1) : le;
+        };
         const uint64_t cmask = (1ull << (2 * a.g.mbits)) - 1ull;
         while (heads) {
-            const uint32_t hd = base + (uint32_t)(__ffs(heads) - 1);
+            const int hl = __ffs(heads) - 1;
             heads &= heads - 1;
-            const uint64_t K = a.skey[hd];
-            uint32_t cs = hd, ce = hd + 1;
-            table_lookup(a.g, K, cs, ce);
-            const int lc = a.lev[hd];
+            const uint64_t K = __shfl_sync(0xffffffffu, key, hl);
+            const uint32_t cs = base + (uint32_t)hl;
+            uint32_t ce = cell_end((uint32_t)hl);
+            const int lc = (int)(K >> (2 * a.g.mbits));
             int span = 1;
             if constexpr (MERGE) {
                 // the following cells of this warp's range join the chunk
@@ -703,13 +782,12 @@ __global__ void __launch_bounds__(128, MERGE ? SPH_TILE_MERGE_BLOCKS : (T == 1 ?
                 // 32 particles
                 const uint32_t fx = compact2(K & cmask), fy = compact2((K & cmask) >> 1);
                 while (ce - cs < 32 && ce < base + 32 && ce < n) {
-                    const uint64_t K2 = a.skey[ce];
+                    const uint64_t K2 = __shfl_sync(0xffffffffu, key, (int)(ce - base));
                     if ((K2 >> (2 * a.g.mbits)) != (K >> (2 * a.g.mbits))) break;
                     const int dx = (int)compact2(K2 & cmask) - (int)fx;
                     const int dy = (int)compact2((K2 & cmask) >> 1) - (int)fy;
                     if (dx < -1 || dx > 1 || dy < -1 || dy > 1) break;
-                    uint32_t s2 = ce, e2 = ce + 1;
-                    table_lookup(a.g, K2, s2, e2);
+                    const uint32_t e2 = cell_end(ce - base);
                     if (e2 - cs > 32) break;
                     heads &= ~(1u << (ce - base));
                     ce = e2;
@@ -717,7 +795,7 @@ __global__ void __launch_bounds__(128, MERGE ? SPH_TILE_MERGE_BLOCKS : (T == 1 ?
                 }
             }
             for (uint32_t p0 = cs; p0 < ce; p0 += 32)
-                tile_chunk<false, 1>(a, sbuf[w], spcs[w], lc, cs, min(ce, p0 + 32), p0, -1,
+                tile_chunk<false, 1>(a, tab, sbuf[w], spcs[w], lc, cs, min(ce, p0 + 32), p0, -1,
                                      span);
         }
     } else {
@@ -731,7 +809,7 @@ __global__ void __launch_bounds__(128, MERGE ? SPH_TILE_MERGE_BLOCKS : (T == 1 ?
             uint32_t cs = t, ce = t + 1;
             table_lookup(a.g, K, cs, ce);
             const uint32_t pe = min(ce, w1);
-            tile_chunk<false, T>(a, sbuf[w], spcs[w], a.lev[t], cs, pe, t, -1);
+            tile_chunk<false, T>(a, tab, sbuf[w], spcs[w], a.lev[t], cs, pe, t, -1);
             t = pe;
         }
     }
@@ -740,17 +818,20 @@ __global__ void __launch_bounds__(128, MERGE ? SPH_TILE_MERGE_BLOCKS : (T == 1 ?
 // Direct-mode pass for the particles whose own entries overflowed their
 // staging row; a warp per queued particle.
 __global__ void __launch_bounds__(128) k_list_tile_queue(ListArgs a) {
-    __shared__ float4 sbuf[4][TILE_CAP];
-    __shared__ int spcs[4][20];
-    const int w = threadIdx.x >> 5;
     const uint32_t nq = *a.nqueue;
+    if (blockIdx.x * 4u >= nq) return;
+    __shared__ float4 sbuf[4][TILE_CAP];
+    __shared__ int spcs[4][TILE_PCS];
+    __shared__ LevTab tab;
+    tab.load(a.g);
+    const int w = threadIdx.x >> 5;
     const uint32_t gw = blockIdx.x * 4u + (uint32_t)w, nw = gridDim.x * 4u;
     for (uint32_t q = gw; q < nq; q += nw) {
         const uint32_t i = a.queue[q];
         // the reference and span of the chunk that queued it
         const uint32_t r = a.qref[q];
         const uint32_t cs = r & 0x7fffffffu;
-        tile_chunk<true, 16>(a, sbuf[w], spcs[w], a.lev[i], cs, i + 1, i, (int)i,
+        tile_chunk<true, 16>(a, tab, sbuf[w], spcs[w], a.lev[i], cs, i + 1, i, (int)i,
                              (r & 0x80000000u) ? 2 : 1);
     }
 }

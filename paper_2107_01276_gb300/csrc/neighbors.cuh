@@ -110,14 +110,11 @@ struct AxisPieces {
     int first[3], last[3], shift[3];
 };
 
-__device__ __forceinline__ bool axis_pieces(const Domain &d, const Level &L,
-                                            const int *bb, int ax, float x,
-                                            float Q, AxisPieces &r) {
-    const int nc = L.n[ax];
-    const int b0 = __ldg(&bb[2 * ax]), b1 = __ldg(&bb[2 * ax + 1]);
+// nc, s, b0, b1: the level's cell count, 1 / cell width and occupied range.
+__device__ __forceinline__ bool axis_pieces_of(bool periodic, int nc, float s, int b0,
+                                               int b1, float x, float Q, AxisPieces &r) {
     // FP32 with a margin far above its rounding ((|x| + Q) / w 2^-21 cells):
     // the pieces only need to cover the exact cell range
-    const float s = L.invw[ax];
     const float margin = (fabsf(x) + Q) * s * (1.0f / 1048576.0f) + (1.0f / 1024.0f);
     const float flo = floorf((x - Q) * s - margin);
     const float fhi = floorf((x + Q) * s + margin);
@@ -127,7 +124,7 @@ __device__ __forceinline__ bool axis_pieces(const Domain &d, const Level &L,
         r.last[k] = 0;
         r.shift[k] = 0;
     }
-    if (d.periodic[ax]) {
+    if (periodic) {
         if (fhi - flo + 1.0f >= (float)nc) {
             r.first[1] = b0;
             r.last[1] = b1;
@@ -148,6 +145,13 @@ __device__ __forceinline__ bool axis_pieces(const Domain &d, const Level &L,
     r.first[1] = flo < (float)b0 ? b0 : (int)flo;
     r.last[1] = fhi > (float)b1 ? b1 : (int)fhi;
     return r.first[1] <= r.last[1];
+}
+
+__device__ __forceinline__ bool axis_pieces(const Domain &d, const Level &L,
+                                            const int *bb, int ax, float x,
+                                            float Q, AxisPieces &r) {
+    return axis_pieces_of(d.periodic[ax], L.n[ax], L.invw[ax], __ldg(&bb[2 * ax]),
+                          __ldg(&bb[2 * ax + 1]), x, Q, r);
 }
 
 // Whether the cells of a query (its axis pieces at level l) meet a block
