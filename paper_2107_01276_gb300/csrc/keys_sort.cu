@@ -422,9 +422,24 @@ __device__ __forceinline__ void radix_small_at(int n, int passes, uint64_t *ka, 
         radix_small_body<uint64_t, RSS_MAX64 / RSS_THREADS>(n, passes, ka, va, cnt, dtot);
 }
 
+// Alone, the sort is compiled for the items a lane really has: the unrolled
+// 16 of the largest sets are many times the instructions that a set of a
+// thousand needs, and their fetching was most of its time.
+template <typename K, int IT>
 __global__ void __launch_bounds__(RSS_THREADS)
     k_radix_small(int n, int passes, uint64_t *ka, uint32_t *va) {
-    radix_small_at(n, passes, ka, va);
+    __shared__ uint32_t cnt[RSS_WARPS][257];
+    __shared__ uint32_t dtot[256];
+    radix_small_body<K, IT>(n, passes, ka, va, cnt, dtot);
+}
+using RadixSmallFn = void (*)(int, int, uint64_t *, uint32_t *);
+static RadixSmallFn radix_small_fn(int n, int passes) {
+    if (passes <= 4)
+        return n <= RSS_THREADS ? k_radix_small<uint32_t, 1>
+               : n <= 4 * RSS_THREADS ? k_radix_small<uint32_t, 4>
+                                      : k_radix_small<uint32_t, RSS_MAX / RSS_THREADS>;
+    return n <= RSS_THREADS ? k_radix_small<uint64_t, 1>
+                            : k_radix_small<uint64_t, RSS_MAX64 / RSS_THREADS>;
 }
 
 // The dynamic shared-memory limit of k_radix_small, raised once per device.
@@ -436,10 +451,15 @@ static bool radix_small_ready() {
         return false;
     }
     if (ok[dev] == 0) {
-        ok[dev] = cudaFuncSetAttribute(k_radix_small,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)radix_small_smem(RSS_MAX, 4)) == cudaSuccess ? 1 : -1;
-        if (ok[dev] < 0) cudaGetLastError();
+        signed char r = 1;
+        for (int passes : {4, 8})
+            for (int n : {RSS_THREADS, 4 * RSS_THREADS, passes == 4 ? RSS_MAX : RSS_MAX64})
+                if (cudaFuncSetAttribute(radix_small_fn(n, passes),
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)radix_small_smem(RSS_MAX, 4)) != cudaSuccess)
+                    r = -1;
+        if (r < 0) cudaGetLastError();
+        ok[dev] = r;
     }
     return ok[dev] == 1;
 }
@@ -453,7 +473,8 @@ void radix_sort(cudaStream_t s, int n, int bits, uint64_t *key,
     if (n <= 1 || bits <= 0) return;
     if (radix_small_takes(n, bits) && radix_small_ready()) {
         const int passes = (bits + 7) / 8;
-        k_radix_small<<<1, RSS_THREADS, radix_small_smem(n, passes), s>>>(n, passes, key, val);
+        radix_small_fn(n, passes)<<<1, RSS_THREADS, radix_small_smem(n, passes), s>>>(
+            n, passes, key, val);
         *launches += 1;
         return;
     }
