@@ -123,6 +123,8 @@ struct sph_ctx {
     int *d_overflow = nullptr;
     uint32_t *longq = nullptr, *d_nlong = nullptr;
     uint32_t *stage = nullptr, *lqueue = nullptr, *d_nlq = nullptr;
+    uint32_t *rlen = nullptr;       // row lengths (ListArgs::rlen)
+    bool rows = false;              // the current lists have rows
     uint32_t *lqref = nullptr;      // queued particles' chunk references
     uint32_t stage_w = 64;          // staging row width (entries)
     uint32_t stage_want = 0;        // width to switch to at the next build
@@ -172,11 +174,11 @@ struct sph_ctx {
 
     bool grid_valid = false, rhs_valid = false, have_dt = false;
     // list sizing: entry total and particle count of the last build that
-    // read its total back, for exact lists and for lists with a skin
-    uint32_t last_total = 0, last_total_skin = 0;
+    // read its total back
+    uint32_t last_total[3] = {};     // per ListForm
     float skin = 1.0f;          // skin factor of the current lists (1: exact)
     int *d_skin_err = nullptr;  // set when particles outran the skin
-    int last_total_n = 0, last_total_skin_n = 0;
+    int last_total_n[3] = {};
     long long steps = 0;
     int launches = 0;
     bool timing = false;
@@ -221,7 +223,14 @@ void pack(sph_ctx *c);
 GatherPackRec gather_pack_rec(sph_ctx *c, bool mid_step);
 bool want_wall_lists(const sph_ctx *c);
 sph_status rebuild(sph_ctx *c, bool mid_step, bool exact = true,
-                          float skin = 1.0f, bool for_walls = true);
+                          float skin = 1.0f, bool for_walls = true, bool rows = false);
+// The list forms whose sizes are remembered apart: exact, with a skin, with
+// a skin and rows.  A build of a form needs no read-back when the last total
+// read back was at most half the list buffer, at a particle count within
+// 10 %.
+enum ListForm { LIST_EXACT, LIST_SKIN, LIST_ROWS };
+ListForm step_form(sph_ctx *c);          // of a step's first build
+bool list_sized(const sph_ctx *c, ListForm f);
 WallBcArgs wall_bc_args(sph_ctx *c);
 void run_passes(sph_ctx *c);
 void run_pec(sph_ctx *c, double f);
@@ -293,6 +302,9 @@ inline PassAArgs<R> pass_a_args(sph_ctx *c) {
     a.an = c->an;
     a.off = c->off;
     a.list = c->list;
+    a.rows = c->rows ? c->stage : nullptr;
+    a.roww = c->stage_w;
+    a.rlen = c->rlen;
     a.pk = c->pk;
     a.x = c->f[F_X];
     a.y = c->f[F_Y];
@@ -332,6 +344,9 @@ inline PassBArgs<R> pass_b_args(sph_ctx *c, const PassAArgs<R> &a) {
     b.an = c->an;
     b.off = c->off;
     b.list = c->list;
+    b.rows = a.rows;
+    b.roww = a.roww;
+    b.rlen = a.rlen;
     b.pk = c->pk;
     b.x = a.x;
     b.y = a.y;

@@ -274,12 +274,7 @@ static bool small_build_ok(sph_ctx *c, float skin) {
     if (!radix_small_available() || want_wall_lists(c) || c->timing) return false;
     if (c->stage_want > c->stage_w) return false;
     if (2 * c->mbits + c->lbits <= 0) return false;
-    const bool sk = skin > 1.0f;
-    const uint32_t lt = sk ? c->last_total_skin : c->last_total;
-    const int ltn = sk ? c->last_total_skin_n : c->last_total_n;
-    if (!(lt > 0 && (size_t)lt * 2 <= c->list_cap && (long long)n * 10 <= (long long)ltn * 11 &&
-          (long long)n * 10 >= (long long)ltn * 9))
-        return false;
+    if (!list_sized(c, skin > 1.0f ? LIST_SKIN : LIST_EXACT)) return false;
     ListArgs la = list_args(c);
     la.skin = skin;
     return list_walk_kind(la) == 1;
@@ -341,6 +336,7 @@ static void plan_small_build(sph_ctx *c, bool mid_step, float skin, bool with_dt
     B.la = list_args(c);
     B.la.skin = skin;
     c->skin = skin;
+    c->rows = false;
     B.scan.in = c->own;
     B.scan.rev = c->rev;
     B.scan.out = c->off;
@@ -539,7 +535,7 @@ static sph_status batch_body(sph_batch *b, const std::vector<sph_ctx *> &all,
         for (int q = a; q < e; ++q) {
             sph_ctx *c = rest[q];
             compute_dt(c, c->d_t, 1);
-            if ((bst[q] = rebuild(c, false, true, is_mixed(c) ? 1.1f : 1.0f)) != SPH_OK) return;
+            if ((bst[q] = rebuild(c, false, true, is_mixed(c) ? 1.1f : 1.0f, true, true)) != SPH_OK) return;
         }
     };
     if (capturing)
@@ -674,14 +670,7 @@ static bool batch_graph_step(sph_batch *b, const std::vector<sph_ctx *> &all,
         if ((uintptr_t)c->s <= 2 && c->s != b->s) return false;
         if (c->stage_want > c->stage_w) return false;
         // each build's list size known with headroom (no read-back)
-        const bool sk = is_mixed(c);
-        const uint32_t lt = sk ? c->last_total_skin : c->last_total;
-        const int ltn = sk ? c->last_total_skin_n : c->last_total_n;
-        const int n = c->n;
-        if (!(lt > 0 && (size_t)lt * 2 <= c->list_cap && (long long)n * 10 <= (long long)ltn * 11 &&
-              (long long)n * 10 >= (long long)ltn * 9))
-            return false;
-        if (!sk && !(c->last_total_n > 0)) return false;
+        if (!list_sized(c, step_form(c))) return false;
     }
     for (sph_ctx *c : all) ensure_set_pk(c, &c->wall);
     std::vector<uintptr_t> key{(uintptr_t)b->s};

@@ -56,17 +56,8 @@ bool graph_step(sph_ctx *c, sph_status *st) {
     }
     if (++c->steps_same_cfg <= 2) return false;
     if (c->stage_want > c->stage_w) return false;
-    {   // the build's list size must be known with headroom (no read-back)
-        const bool sk = is_mixed(c);
-        const uint32_t lt = sk ? c->last_total_skin : c->last_total;
-        const int ltn = sk ? c->last_total_skin_n : c->last_total_n;
-        const int n = c->n;
-        if (!(lt > 0 && (size_t)lt * 2 <= c->list_cap &&
-              (long long)n * 10 <= (long long)ltn * 11 &&
-              (long long)n * 10 >= (long long)ltn * 9))
-            return false;
-        if (!is_mixed(c) && !(c->last_total_n > 0)) return false;
-    }
+    // the build's list size must be known with headroom (no read-back)
+    if (!list_sized(c, step_form(c))) return false;
     ensure_set_pk(c, &c->wall);
     const std::vector<uintptr_t> key = graph_key(c);
     sph_ctx::StepGraph *g = nullptr;
@@ -92,6 +83,7 @@ bool graph_step(sph_ctx *c, sph_status *st) {
         int64_t *id0 = c->id, *ida0 = c->id_alt;
         const uint32_t tmask0 = c->tmask;
         const float skin0 = c->skin;
+        const bool rows0 = c->rows;
         const long long steps0 = c->steps;
         const bool gv0 = c->grid_valid, rv0 = c->rhs_valid;
         const int l0 = c->launches;
@@ -117,6 +109,7 @@ bool graph_step(sph_ctx *c, sph_status *st) {
             c->id_alt = ida0;
             c->tmask = tmask0;
             c->skin = skin0;
+            c->rows = rows0;
             c->steps = steps0;
             c->grid_valid = gv0;
             c->rhs_valid = rv0;

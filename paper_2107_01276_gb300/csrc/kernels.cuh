@@ -124,11 +124,12 @@ __device__ __forceinline__ void qs_ws(double q, double &w, double &s) {
 // x != 0 for x >= 0, on the integer pipe
 __device__ __forceinline__ bool nonzero(double x) { return __double_as_longlong(x) != 0; }
 
-// Mixed pair sums of sets without walls (LEAN): bound by instruction issue,
-// not by the FP32 pipe (pass B at 16.8M: ~165 thread instructions a pair,
-// 90 flop), so two values share an instruction where the formulas come in
-// pairs: the axes of a separation, u and v, the kernels of h_i and h_j.
-// Each half rounds like the scalar operation.
+// Mixed pair sums of sets without walls (LEAN): two values share an
+// instruction where the formulas come in pairs: the axes of a separation, u
+// and v, the kernels of h_i and h_j.  Each half rounds like the scalar
+// operation.  At 1M particles of the 1:250 strip pass B issues 215M warp
+// instructions and is bound by issue (72 % busy) and by the L1 data pipe of
+// its record gathers (85 %).
 struct F2 {
     unsigned long long v;
 };

@@ -265,6 +265,27 @@ __global__ void __launch_bounds__(128) k_list_place(ListArgs a) {
     list_place_at<T>(a, i, tm);
 }
 
+// Rows: only the reverse entries are placed (the coarser entries of each
+// row).  A thread per particle; most rows have none.  4.2M graded strip:
+// walk to sorted lists but for the walk itself 1.16 -> 0.57 ms, where
+// k_list_place copied every row into the lists; and the passes, which read
+// 32 separate lists a warp before, 1.155 -> 0.935 ms (B) and 0.935 -> 0.92
+// ms (A).
+__global__ void __launch_bounds__(256) k_list_place_rev(ListArgs a) {
+    const uint32_t i = blockIdx.x * 256 + threadIdx.x;
+    if (i < (uint32_t)a.n) {
+        const uint32_t r = a.rlen[i], e = r & 0xffffu;
+        const uint32_t *row = a.stage + (size_t)(i >> 5) * (32 * a.stage_w) + (i & 31);
+        for (uint32_t k = r >> 16; k < e; ++k) {
+            const uint32_t j = row[32 * k];
+            if (!SPH_DCHECK(j < (uint32_t)a.n)) continue;
+            const uint32_t rp = a.off[j] + a.own[j] + atomicAdd(&a.rev[j], 1u);
+            if (rp < a.cap) a.list[rp] = i;
+        }
+        if (i == (uint32_t)a.n - 1 && a.off[a.n] > a.cap) atomicOr(a.overflow, 1);
+    }
+}
+
 // Second walk for the queued particles (more than stage_w own entries):
 // same order as k_list_gather; teams take queue entries in turn.
 template <int T>
@@ -414,7 +435,8 @@ __device__ __forceinline__ float box_gap2(const Domain &d, const LevTab &T, int 
 // error analysis grows with it.  A particle queued for the direct pass
 // records its chunk's reference and span, so that pass takes the same
 // decisions with the same arithmetic.
-template <bool DIRECT, int T>
+// ROWS: interleaved rows (ListArgs::rows), else one after another.
+template <bool DIRECT, int T, bool ROWS = false>
 __device__ __forceinline__ void tile_chunk(const ListArgs &a, const LevTab &tab,
                                            float4 *sc, int *pcs, int lc, uint32_t cs,
                                            uint32_t pe, uint32_t p0, int only,
@@ -448,9 +470,10 @@ __device__ __forceinline__ void tile_chunk(const ListArgs &a, const LevTab &tab,
     const float bx = 0.5f * (rxhi - rxlo), by = 0.5f * (ryhi - rylo);
     const float Rmx = a.skin * (3.0f * hmx);   // largest pair radius of a chunk particle
     const uint32_t W = a.stage_w;
-    uint32_t k = 0;
+    constexpr uint32_t RS = ROWS ? 32 : 1;     // stride of a row's entries
+    uint32_t k = 0, kown = 0;
     if (DIRECT && act) k = a.off[i];
-    uint32_t *row = a.stage + (size_t)i * W;
+    uint32_t *row = a.stage + (ROWS ? (size_t)(i >> 5) * (32 * W) + (i & 31) : (size_t)i * W);
     const float Amax = fmaxf(a.an.A[0], a.an.A[1]);
     const float Lx = (float)a.d.L[0], Ly = (float)a.d.L[1];
     const float iLx = 1.0f / Lx, iLy = 1.0f / Ly;
@@ -674,7 +697,8 @@ __device__ __forceinline__ void tile_chunk(const ListArgs &a, const LevTab &tab,
                                 if (DIRECT) {
                                     if (in) put(k, ent);
                                 } else {
-                                    if (in && k < W) row[k] = ent;
+                                    if (in && k < W)
+                                        row[k * RS] = ROWS && CO ? ent & ~STAGE_COARSE : ent;
                                     if (CO && in) atomicAdd(&a.rev[ent & ~STAGE_COARSE], 1u);
                                 }
                                 k += in ? 1u : 0u;
@@ -697,6 +721,7 @@ __device__ __forceinline__ void tile_chunk(const ListArgs &a, const LevTab &tab,
                     using FF = std::false_type;
                     auto both = [&](auto ex, auto wr) {
                         test(ex, wr, FF(), 0u, mf);
+                        if (ROWS && mf) kown = k;
                         if (mf < m) test(ex, wr, TT(), mf, m);
                     };
                     if (exact) {
@@ -714,7 +739,8 @@ __device__ __forceinline__ void tile_chunk(const ListArgs &a, const LevTab &tab,
 #pragma unroll
         for (int o = 16; o; o >>= 1) km = max(km, __shfl_xor_sync(0xffffffffu, km, o));
         if (act && sub == 0) {
-            a.own[i] = k;
+            if (ROWS) a.rlen[i] = k > W ? 0u : k | (kown << 16);
+            a.own[i] = ROWS && k <= W ? 0u : k;
             if (k > W) {
                 const uint32_t q = atomicAdd(a.nqueue, 1u);
                 a.queue[q] = i;
@@ -737,7 +763,7 @@ __device__ __forceinline__ void tile_chunk(const ListArgs &a, const LevTab &tab,
 #ifndef SPH_TILE_MERGE_BLOCKS
 #define SPH_TILE_MERGE_BLOCKS 6
 #endif
-template <int T, bool MERGE = false>
+template <int T, bool MERGE = false, bool ROWS = false>
 __global__ void __launch_bounds__(128, MERGE ? SPH_TILE_MERGE_BLOCKS : (T == 1 ? 7 : 6))
     k_list_tile(ListArgs a) {
     __shared__ float4 sbuf[4][TILE_CAP];
@@ -795,8 +821,8 @@ __global__ void __launch_bounds__(128, MERGE ? SPH_TILE_MERGE_BLOCKS : (T == 1 ?
                 }
             }
             for (uint32_t p0 = cs; p0 < ce; p0 += 32)
-                tile_chunk<false, 1>(a, tab, sbuf[w], spcs[w], lc, cs, min(ce, p0 + 32), p0, -1,
-                                     span);
+                tile_chunk<false, 1, ROWS>(a, tab, sbuf[w], spcs[w], lc, cs,
+                                           min(ce, p0 + 32), p0, -1, span);
         }
     } else {
         constexpr uint32_t P = 32 / T;
@@ -1055,6 +1081,9 @@ static int walk_kind(const ListArgs &a) {
 }
 
 int list_walk_kind(const ListArgs &a) { return walk_kind(a); }
+// The merged walk's range, whatever walk is set: below it a step is bound by
+// launches and the copy into the lists is small.
+bool list_rows_for(const ListArgs &a) { return a.n >= 48000 && walk_kind(a) == 4; }
 int list_place_team(int n) { return std::max(team_size(n), 16); }
 int fill_queue_blocks() { return 4; }
 int sort_long_blocks(int n) { return std::max(1, std::min(8, nblk(n, 4))); }
@@ -1110,7 +1139,10 @@ void launch_list_walk(cudaStream_t s, const ListArgs &a, int *launches) {
     if (kind == 3) {
         k_list_tile<1><<<nblk(n, 128), 128, 0, s>>>(a);
     } else if (kind == 4) {
-        k_list_tile<1, true><<<nblk(n, 128), 128, 0, s>>>(a);
+        if (a.rows)
+            k_list_tile<1, true, true><<<nblk(n, 128), 128, 0, s>>>(a);
+        else
+            k_list_tile<1, true><<<nblk(n, 128), 128, 0, s>>>(a);
     } else if (kind == 2) {
         k_list_tile<4><<<nblk(n, 32), 128, 0, s>>>(a);
     } else {
@@ -1138,10 +1170,13 @@ void build_lists_fill(cudaStream_t s, ListArgs a, bool mixed, bool queue,
     if (n <= 0) return;
     // at least 16 lanes per particle: a list's entries are then read from
     // the staging row and written to the list in 64-byte runs
-    with_team(n, [&](auto t) {
-        constexpr int T = decltype(t)::value;
-        k_list_place<T><<<nblk(n * T, 128), 128, 0, s>>>(a);
-    }, 16);
+    if (a.rows)
+        k_list_place_rev<<<nblk(n, 256), 256, 0, s>>>(a);
+    else
+        with_team(n, [&](auto t) {
+            constexpr int T = decltype(t)::value;
+            k_list_place<T><<<nblk(n * T, 128), 128, 0, s>>>(a);
+        }, 16);
     if (queue) {
         if (walk_kind(a) != 1)
             k_list_tile_queue<<<152 * 4, 128, 0, s>>>(a);

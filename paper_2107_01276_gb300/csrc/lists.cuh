@@ -62,6 +62,15 @@ struct ListArgs {
     // (a superset of N(i) for particles that move less than the skin
     // allows); 1: exactly N(i)
     float skin;
+    // rows (merged-chunk walk only): the passes read own entries from the
+    // staging rows, which are interleaved by 32 particles (entry k of i at
+    // [i / 32][k][i % 32]: a warp's loads of its k-th entries are one line);
+    // the lists hold reverse entries, and the own entries of the particles
+    // whose rows overflowed, whose count own[i] is then (zero for the
+    // others)
+    bool rows;
+    uint32_t *rlen;             // rows: entries of i's row | those on its own
+                                // level << 16 (they come first)
     // walk: 1 per-particle team walk, 2 cell tiles with 4-lane teams, 3
     // cell tiles with a lane per particle, 4 the same with neighbouring
     // cells of a level merged into one chunk while they hold at most 32
@@ -93,6 +102,7 @@ struct SortSegRec {
     uint32_t cap;
     uint32_t *longq, *nlong;
 };
+bool list_rows_for(const ListArgs &a);   // whether the size rule takes rows
 int list_walk_kind(const ListArgs &a);   // 1 team walk, 2 / 3 cell tiles
 int list_place_team(int n);              // lanes per particle of the placement
 int fill_queue_blocks();

@@ -13,31 +13,33 @@
 
 namespace sph {
 
-// List entries whose neighbour records a mixed-path pass loads ahead.
-#ifndef SPH_UNROLL_A
-#define SPH_UNROLL_A 4
-#endif
-#ifndef SPH_UNROLL_B
-#define SPH_UNROLL_B 2
-#endif
-constexpr int UNROLL_A = SPH_UNROLL_A;
-constexpr int UNROLL_B = SPH_UNROLL_B;
+// List entries whose neighbour records a mixed-path pass loads together (the
+// next ones' indices are on their way meanwhile).  One lane a particle:
+// measured at 4.2M on the 1:250 strip at seven resident blocks, pass A 2, 3,
+// 4 entries 0.99, 0.92, 0.93 ms, pass B 1, 2, 3 entries (eight, seven, five
+// blocks) 1.42, 0.93, 1.04 ms.  Teams have few iterations: 26k particles,
+// pass A 2, 3 entries 16.5, 19.8 us, pass B 1, 2 entries 19.0, 20.4 us.
+template <int T>
+constexpr int UNROLL_A = T == 1 ? 3 : 2;
+template <int T>
+constexpr int UNROLL_B = T == 1 ? 2 : 1;
 
 // Membership test of a list entry when the lists carry a skin: the exact
 // predicate of N(i) on the separation the pass already has (FP32 band test
-// with the FP64 predicate inside the band on the mixed path; the FP64
-// predicate on the FP64 path).
-template <typename R>
-__device__ __forceinline__ bool skin_member(const Domain &d, const Anchor &an,
-                                            R r2, R hi, R hj, double xi,
-                                            double yi, double hid,
-                                            const double *x, const double *y,
-                                            const double *h, int j) {
+// with the FP64 predicate inside the band on the mixed path, which alone
+// reads i's FP64 values; the FP64 predicate on the FP64 path).
+template <typename R, class Args>
+__device__ __forceinline__ bool skin_member(const Args &a, R r2, R hi, R hj, int i, int j) {
     if constexpr (sizeof(R) == 4) {
-        return member_r2(d, an, r2, hi, hj, xi, yi, hid, x, y, h, j);
-    } else {
-        return pred_fp64(d, xi, yi, hid, __ldg(&x[j]), __ldg(&y[j]), __ldg(&h[j]));
+        const float R1 = 3.0f * fmaxf(hi, hj);
+        const float R2 = R1 * R1;
+        const float band = (R2 + 4.0f * fmaxf(a.an.A[0], a.an.A[1]) * R1) *
+                           (1.0f / 65536.0f);
+        if (r2 < R2 - band) return true;
+        if (r2 > R2 + band) return false;
     }
+    return pred_fp64(a.d, __ldg(&a.x[i]), __ldg(&a.y[i]), __ldg(&a.h[i]), __ldg(&a.x[j]),
+                     __ldg(&a.y[j]), __ldg(&a.h[j]));
 }
 
 // ---------------------------------------------------------------- pass A --
@@ -403,16 +405,35 @@ struct PassBLane {
     }
 };
 
-// Pass A over the list entries [b, e) of particle i, in list order (team
-// lane t takes entries b + t, b + t + T, ...).
+// The entries of particle i: its row, if the lists have rows, and its list
+// behind it, as one sequence (a particle next to a finer level has few row
+// entries and many list entries: two loops would each take the warp's
+// longest, a third more instructions on the 1:250 strip).
+struct Entries {
+    const uint32_t *row, *list;   // list: entry k at list[k]
+    uint32_t nr, cnt;
+    template <class Args>
+    __device__ __forceinline__ Entries(const Args &a, int i) {
+        nr = a.rows ? __ldg(&a.rlen[i]) & 0xffffu : 0u;
+        row = a.rows + ((size_t)(i >> 5) * (32 * a.roww) + (i & 31));
+        const uint32_t b = __ldg(&a.off[i]);
+        cnt = __ldg(&a.off[i + 1]) - b + nr;
+        list = a.list + ((ptrdiff_t)b - (ptrdiff_t)nr);
+    }
+    __device__ __forceinline__ int at(uint32_t k, int i) const {
+        const uint32_t *p = k < nr ? row : list;
+        return k < cnt ? (int)__ldg(&p[k < nr ? 32 * k : k]) : i;
+    }
+};
+
+// Pass A over the entries of particle i, in order (team lane t takes entries
+// t, t + T, ...).
 template <typename R, int T, bool LEAN>
 __device__ __forceinline__ void pass_a_list(const PassAArgs<R> &a, int i,
-                                            PassALane<R, LEAN> &L, const Team<T> &tm,
-                                            uint32_t b, uint32_t e) {
+                                            PassALane<R, LEAN> &L, const Team<T> &tm) {
     Sep<R> sp;
     sp.init(a.d, a.x, a.y, a.pk, i);
     const R hi = L.hi;
-    const double xid = a.x[i], yid = a.y[i], hid = a.h[i];
     if constexpr (sizeof(R) == 4) {
         // U list entries per step, their records loaded before any is used
         // (more loads in flight per warp)
@@ -423,73 +444,73 @@ __device__ __forceinline__ void pass_a_list(const PassAArgs<R> &a, int i,
                 // r = 0 (i itself): the gradient sums add zero by s = 0, d = 0
                 const F2 d = sp2.get(pj);
                 const R r2 = fmaf(lo(d), lo(d), sph::hi(d) * sph::hi(d));
-                const bool in = !a.filter || skin_member<R>(a.d, a.an, r2, hi, pj.z, xid,
-                                                            yid, hid, a.x, a.y, a.h, j);
+                const bool in = !a.filter || skin_member<R>(a, r2, hi, pj.z, i, j);
                 L.pair2(mj, pj.z, pjv, in, d, r2, acc);
                 return;
             }
             R dx, dy;
             anchor_sep(a.an, sp.pi, pj, dx, dy);
             const R r2 = fmaf(dx, dx, dy * dy);
-            if (a.filter && !skin_member<R>(a.d, a.an, r2, hi, pj.z, xid, yid,
-                                            hid, a.x, a.y, a.h, j))
+            if (a.filter && !skin_member<R>(a, r2, hi, pj.z, i, j))
                 return;
             L.pair(mj, pj.z, pjv, j == i, dx, dy, r2);
         };
-        constexpr int U = UNROLL_A;
-        uint32_t k = b + tm.lane;
-        for (; k + (U - 1) * T < e; k += U * T) {
+        constexpr int U = UNROLL_A<T>;
+        const Entries E(a, i);
+        uint32_t k = tm.lane;
+        int jn[U];   // the next entries, loaded ahead of their records
+#pragma unroll
+        for (int u = 0; u < U; ++u) jn[u] = E.at(k + u * T, i);
+        for (; k + (U - 1) * T < E.cnt; k += U * T) {
             int jj[U];
             float4 pp[U];
             R mm[U], qq[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                jj[u] = (int)__ldg(&a.list[k + u * T]);
+                jj[u] = jn[u];
                 // an index out of range (debug builds) reads i instead
                 if (!SPH_DCHECK((unsigned)jj[u] < (unsigned)a.n)) jj[u] = i;
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
                 pp[u] = __ldg(&a.pk[jj[u]]);
                 mm[u] = a.m[jj[u]];
                 qq[u] = a.p[jj[u]];
             }
 #pragma unroll
+            for (int u = 0; u < U; ++u) jn[u] = E.at(k + (U + u) * T, i);
+#pragma unroll
             for (int u = 0; u < U; ++u) body(jj[u], pp[u], mm[u], qq[u]);
         }
-        for (; k < e; k += T) {
-            int j = (int)__ldg(&a.list[k]);
-            if (!SPH_DCHECK((unsigned)j < (unsigned)a.n)) j = i;
-            body(j, __ldg(&a.pk[j]), a.m[j], a.p[j]);
+#pragma unroll
+        for (int u = 0; u < U - 1; ++u) {
+            if (k + u * T >= E.cnt) break;
+            if (!SPH_DCHECK((unsigned)jn[u] < (unsigned)a.n)) jn[u] = i;
+            body(jn[u], __ldg(&a.pk[jn[u]]), a.m[jn[u]], a.p[jn[u]]);
         }
         if constexpr (LEAN) {
             L.ax = lo(acc);
             L.ay = sph::hi(acc);
         }
     } else {
-        for (uint32_t k = b + tm.lane; k < e; k += T) {
-            const int j = (int)__ldg(&a.list[k]);
+        const Entries E(a, i);   // FP64 steps take exact lists: no rows
+        for (uint32_t k = tm.lane; k < E.cnt; k += T) {
+            const int j = (int)__ldg(&E.list[k]);
             if (!SPH_DCHECK((unsigned)j < (unsigned)a.n)) continue;
             R dx, dy, r2, hj;
             sp.get(a.d, a.an, a.x, a.y, a.h, a.pk, j, dx, dy, r2, hj);
-            if (a.filter && !skin_member<R>(a.d, a.an, r2, hi, hj, xid, yid, hid,
-                                            a.x, a.y, a.h, j))
+            if (a.filter && !skin_member<R>(a, r2, hi, hj, i, j))
                 continue;
             L.pair(a.m[j], hj, a.p[j], j == i, dx, dy, r2);
         }
     }
 }
 
-// Pass B over the list entries [b, e) of particle i, in list order.
+// Pass B over the entries of particle i, in order.
 template <typename R, int T, bool LEAN>
 __device__ __forceinline__ void pass_b_list(const PassBArgs<R> &a, int i,
-                                            PassBLane<R, LEAN> &L, const Team<T> &tm,
-                                            uint32_t b, uint32_t e) {
+                                            PassBLane<R, LEAN> &L, const Team<T> &tm) {
     Sep<R> sp;
     sp.init(a.d, a.x, a.y, a.pk, i);
     const R pavg_i = L.pavg_i;
     const bool literal = a.pavg_mode != 0;
-    const double xid = a.x[i], yid = a.y[i], hid = a.h[i];
     const R hpk = (R)a.pk[i].z;   // h_i as the list builder saw it
     if constexpr (sizeof(R) == 4) {
         // neither a membership test for skin entries nor a test for i
@@ -509,42 +530,47 @@ __device__ __forceinline__ void pass_b_list(const PassBArgs<R> &a, int i,
             L.pair_rec(dx, dy, fmaf(dx, dx, dy * dy), A, B,
                        literal ? a.pavg[j] : pavg_i);
         };
-        constexpr int U = UNROLL_B;
-        uint32_t k = b + tm.lane;
-        for (; k + (U - 1) * T < e; k += U * T) {
+        constexpr int U = UNROLL_B<T>;
+        const Entries E(a, i);
+        uint32_t k = tm.lane;
+        int jn[U];   // the next entries, loaded ahead of their records
+#pragma unroll
+        for (int u = 0; u < U; ++u) jn[u] = E.at(k + u * T, i);
+        for (; k + (U - 1) * T < E.cnt; k += U * T) {
             int jj[U];
             float4 pp[U], AA[U], BB[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                jj[u] = (int)__ldg(&a.list[k + u * T]);
+                jj[u] = jn[u];
+                // an index out of range (debug builds) reads i instead
                 if (!SPH_DCHECK((unsigned)jj[u] < (unsigned)a.n)) jj[u] = i;
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
                 pp[u] = __ldg(&a.pk[jj[u]]);
                 AA[u] = a.nbA[jj[u]];
                 BB[u] = a.nbB[jj[u]];
             }
 #pragma unroll
+            for (int u = 0; u < U; ++u) jn[u] = E.at(k + (U + u) * T, i);
+#pragma unroll
             for (int u = 0; u < U; ++u) body(jj[u], pp[u], AA[u], BB[u]);
         }
-        for (; k < e; k += T) {
-            int j = (int)__ldg(&a.list[k]);
-            if (!SPH_DCHECK((unsigned)j < (unsigned)a.n)) j = i;
-            body(j, __ldg(&a.pk[j]), a.nbA[j], a.nbB[j]);
+#pragma unroll
+        for (int u = 0; u < U - 1; ++u) {
+            if (k + u * T >= E.cnt) break;
+            if (!SPH_DCHECK((unsigned)jn[u] < (unsigned)a.n)) jn[u] = i;
+            body(jn[u], __ldg(&a.pk[jn[u]]), a.nbA[jn[u]], a.nbB[jn[u]]);
         }
         if constexpr (LEAN) L.take(S);
     } else {
-        for (uint32_t k = b + tm.lane; k < e; k += T) {
-            const int j = (int)__ldg(&a.list[k]);
+        const Entries E(a, i);   // FP64 steps take exact lists: no rows
+        for (uint32_t k = tm.lane; k < E.cnt; k += T) {
+            const int j = (int)__ldg(&E.list[k]);
             if (!SPH_DCHECK((unsigned)j < (unsigned)a.n)) continue;
             if (j == i) continue;
             R dx, dy, r2;
             if (a.filter) {
                 R hj;
                 sp.get(a.d, a.an, a.x, a.y, a.h, a.pk, j, dx, dy, r2, hj);
-                if (!skin_member<R>(a.d, a.an, r2, hpk, hj, xid, yid, hid, a.x,
-                                    a.y, a.h, j))
+                if (!skin_member<R>(a, r2, hpk, hj, i, j))
                     continue;
             } else {
                 sp.get(a.d, a.an, a.x, a.y, a.pk, j, dx, dy, r2);

@@ -19,18 +19,13 @@
 
 namespace sph {
 
-// resident 128-thread blocks per SM the mixed passes are compiled for
-#ifndef SPH_PASS_A_BLOCKS
-#define SPH_PASS_A_BLOCKS 8
-#endif
-#ifndef SPH_PASS_B_BLOCKS
-#define SPH_PASS_B_BLOCKS 8
-#endif
-constexpr int PASS_A_BLOCKS = SPH_PASS_A_BLOCKS;
-constexpr int PASS_B_BLOCKS = SPH_PASS_B_BLOCKS;
+// resident 128-thread blocks per SM the mixed one-lane passes are compiled
+// for (72 registers; at eight, 64 registers, pass B takes 1.50 instead of
+// 0.93 ms at 4.2M, at six 0.94)
+constexpr int PASS_A_BLOCKS = 7;
+constexpr int PASS_B_BLOCKS = 7;
 // Team forms (T > 1: small and walled sets) and the batched forms keep six
-// and five blocks (80 / 96 registers): at the eight-block cap their wall
-// loops spill.
+// and five blocks (80 / 96 registers), for their wall loops.
 template <typename R, int T>
 constexpr int pass_blocks(int lane1) {
     return sizeof(R) == 4 ? (T == 1 ? lane1 : 6) : 1;
@@ -47,7 +42,7 @@ __device__ __forceinline__ void pass_a_at(const PassAArgs<R> &a, int i,
                                           const Team<T> &tm) {
     PassALane<R, !WALLS> L;
     L.init(a, i);
-    pass_a_list<R, T, !WALLS>(a, i, L, tm, a.off[i], a.off[i + 1]);
+    pass_a_list<R, T, !WALLS>(a, i, L, tm);
     if constexpr (WALLS) L.walls(a, i, tm);
     L.finish(a, i, tm);
 }
@@ -63,9 +58,6 @@ __global__ void __launch_bounds__(128, (pass_blocks<R, T>(PASS_A_BLOCKS)))
 
 // ---------------------------------------------------------------- pass B --
 // Pass B of particle i over its list (arithmetic in PassBLane).
-// (float, one lane per particle: at most 64 registers, eight 128-thread
-// blocks per SM, measured faster than six at 80 registers on the graded
-// 1:250 strip)
 template <typename R, int T, bool WALLS>
 __device__ __forceinline__ void pass_b_at(const PassBArgs<R> &a, int i,
                                           const Team<T> &tm) {
@@ -78,7 +70,7 @@ __device__ __forceinline__ void pass_b_at(const PassBArgs<R> &a, int i,
         }
         return;
     }
-    pass_b_list<R, T, !WALLS>(a, i, L, tm, a.off[i], a.off[i + 1]);
+    pass_b_list<R, T, !WALLS>(a, i, L, tm);
     if constexpr (WALLS) L.walls(a, i, tm);
     L.finish(a, i, tm, true);
 }

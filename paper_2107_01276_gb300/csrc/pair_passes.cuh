@@ -16,6 +16,9 @@ struct PassAArgs {
     Domain d;
     Anchor an;
     const uint32_t *off, *list;  // CSR neighbour lists
+    // own entries in interleaved rows before those (ListArgs::rows), or NULL
+    const uint32_t *rows, *rlen;
+    uint32_t roww;
     const float4 *pk;          // anchor coordinates (mixed path)
     const double *x, *y, *h;   // FP64 positions and smoothing lengths
     const R *m, *p, *u, *v;    // pair-arithmetic copies
@@ -34,7 +37,8 @@ struct PassBArgs {
     int n;
     Domain d;
     Anchor an;
-    const uint32_t *off, *list;
+    const uint32_t *off, *list, *rows, *rlen;
+    uint32_t roww;
     const float4 *pk;
     const double *x, *y, *h;
     const R *m, *p, *u, *v;

@@ -121,9 +121,14 @@ Grid grid_for_kernels(const sph_ctx *c) {
 // Keys, stable sort, gather of the state in sorted order, cell table and
 // (mixed path) float mirrors.  mid_step: also carry the PEC stage-start
 // copies x0..p0.
+// staging rows of whole groups of 32 particles (ListArgs::rows)
+static size_t stage_elems(size_t n, uint32_t w) { return (n + 31) / 32 * 32 * w; }
+
 ListArgs list_args(sph_ctx *c) {
     ListArgs la;
     la.skin = 1.0f;
+    la.rows = false;
+    la.rlen = c->rlen;
     la.n = c->n;
     la.g = grid_for_kernels(c);
     la.d = c->dom;
@@ -236,21 +241,30 @@ bool want_wall_lists(const sph_ctx *c) {
     return c->wall.n >= 2048;
 }
 
+ListForm step_form(sph_ctx *c) {
+    if (!is_mixed(c)) return LIST_EXACT;
+    return list_rows_for(list_args(c)) ? LIST_ROWS : LIST_SKIN;
+}
+
+bool list_sized(const sph_ctx *c, ListForm f) {
+    const long long n = c->n, ltn = c->last_total_n[f];
+    return c->last_total[f] > 0 && (size_t)c->last_total[f] * 2 <= c->list_cap &&
+           n * 10 <= ltn * 11 && n * 10 >= ltn * 9;
+}
+
+// rows: the lists serve the pair passes only, which take own entries from
+// the staging rows where the size rule says so.
 sph_status rebuild(sph_ctx *c, bool mid_step, bool exact,
-                   float skin, bool for_walls) {
+                   float skin, bool for_walls, bool rows) {
     const int n = c->n;
     const bool sk = skin > 1.0f;
-    const uint32_t lt = sk ? c->last_total_skin : c->last_total;
-    const int ltn = sk ? c->last_total_skin_n : c->last_total_n;
-    if (exact && lt > 0 && (size_t)lt * 2 <= c->list_cap &&
-        (long long)n * 10 <= (long long)ltn * 11 &&
-        (long long)n * 10 >= (long long)ltn * 9)
-        exact = false;
+    const ListForm form = rows && sk ? step_form(c) : sk ? LIST_SKIN : LIST_EXACT;
+    if (exact && list_sized(c, form)) exact = false;
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     cudaStreamIsCapturing(c->s, &capturing);
     if (c->stage_want > c->stage_w && capturing == cudaStreamCaptureStatusNone) {
         uint32_t *ns = nullptr;
-        if (dalloc(&ns, (size_t)c->cap * c->stage_want, c->s)) {
+        if (dalloc(&ns, stage_elems(c->cap, c->stage_want), c->s)) {
             dfree(c->stage, c->s);   // after the last build's use of it, in stream order
             c->stage = ns;
             c->stage_w = c->stage_want;
@@ -289,7 +303,9 @@ sph_status rebuild(sph_ctx *c, bool mid_step, bool exact,
     t_end(c, 6, es);
     ListArgs la = list_args(c);
     la.skin = skin;
+    la.rows = form == LIST_ROWS;
     c->skin = skin;
+    c->rows = la.rows;
     {
         cudaEvent_t ew;
         t_begin(c, 5, &ew);
@@ -340,13 +356,8 @@ sph_status rebuild(sph_ctx *c, bool mid_step, bool exact,
             wa.cap = c->wcap;
             c->cfg_version += 1;
         }
-        if (sk) {
-            c->last_total_skin = total;
-            c->last_total_skin_n = n;
-        } else {
-            c->last_total = total;
-            c->last_total_n = n;
-        }
+        c->last_total[form] = std::max(total, 1u);   // 0: not known
+        c->last_total_n[form] = n;
         // widen the staging rows from the next build on, so that particles
         // rarely take the second walk (at most 256 entries a row)
         queue = max_own > c->stage_w;
@@ -369,6 +380,7 @@ sph_status rebuild(sph_ctx *c, bool mid_step, bool exact,
             c->list_cap = want;
             la = list_args(c);
             la.skin = skin;
+            la.rows = form == LIST_ROWS;
         }
     }
     build_lists_fill(c->s, la, is_mixed(c), queue, &c->launches);
@@ -506,7 +518,7 @@ void free_ctx(sph_ctx *c) {
                   c->tkey, c->tstart, c->tend, c->tmaxh, c->bbox, c->level_mask,
                   c->d_dt, c->d_t, c->d_hmin, c->d_nonfinite,
                   c->d_total, c->lvl, c->pk, c->own, c->rev, c->off, c->list,
-                  c->d_overflow, c->d_skin_err, c->longq, c->d_nlong, c->stage, c->lqueue, c->lqref, c->d_max_own,
+                  c->d_overflow, c->d_skin_err, c->longq, c->d_nlong, c->stage, c->rlen, c->lqueue, c->lqref, c->d_max_own,
                   c->d_nlq, c->tmp_a, c->tmp_b,
                   c->closest, c->mh0, c->mds, c->mq, c->d_mass, c->d_mass_part, c->wp, c->wugx,
                   c->wugy, c->d_aux, c->d_load};
@@ -879,7 +891,7 @@ sph_status new_ctx(const sph_params *p, cudaStream_t stream, bool has_ds,
     ok = ok && dalloc(&c->lvl, N, c->s) && dalloc(&c->pk, N, c->s) && dalloc(&c->own, N, c->s) &&
          dalloc(&c->rev, N, c->s) && dalloc(&c->off, N + 1, c->s) &&
          dalloc(&c->longq, N, c->s) && dalloc(&c->d_nlong, 1, c->s) &&
-         dalloc(&c->stage, N * c->stage_w, c->s) && dalloc(&c->lqueue, N, c->s) && dalloc(&c->lqref, N, c->s) &&
+         dalloc(&c->stage, stage_elems(N, c->stage_w), c->s) && dalloc(&c->rlen, N, c->s) && dalloc(&c->lqueue, N, c->s) && dalloc(&c->lqref, N, c->s) &&
          dalloc(&c->d_nlq, 1, c->s) && dalloc(&c->d_max_own, 1, c->s);
     ok = ok && dalloc(&c->tmp_a, N + 1, c->s) && dalloc(&c->tmp_b, N + 1, c->s) &&
          dalloc(&c->closest, N, c->s) && dalloc(&c->mh0, N, c->s) && dalloc(&c->mds, N, c->s) &&
@@ -988,7 +1000,7 @@ sph_status check_overflow(sph_ctx *c, const char *who) {
     }
     if (!flags[0]) return SPH_OK;
     cudaMemsetAsync(c->d_overflow, 0, sizeof(int), c->s);
-    c->last_total = c->last_total_skin = 0;   // next builds size exactly
+    memset(c->last_total, 0, sizeof(c->last_total));   // next builds size exactly
     return fail(c, SPH_ECAPACITY, std::string(who) + ": neighbour list overflow");
 }
 
@@ -1025,7 +1037,7 @@ static void forces_launch(sph_ctx *c) {
 sph_status pec_step(sph_ctx *c, bool exact) {
     const float step_skin = is_mixed(c) ? 1.1f : 1.0f;
     compute_dt(c, c->d_t, 1);
-    sph_status st = rebuild(c, false, exact, step_skin);
+    sph_status st = rebuild(c, false, exact, step_skin, true, true);
     if (st != SPH_OK) return st;
     run_passes(c);
     run_pec(c, 0.5);   // (mixed: and the records of the predicted state)
@@ -1416,7 +1428,7 @@ static sph_status read_field(sph_ctx *c, sph_field field, void *dst, long long c
         cudaMemcpyAsync(&ovf, c->d_overflow, sizeof(int), cudaMemcpyDeviceToHost, c->s);
         if (cudaStreamSynchronize(c->s) != cudaSuccess) return cuda_check(c, "sph_read");
         if (ovf) {
-            c->last_total = c->last_total_skin = 0;
+            memset(c->last_total, 0, sizeof(c->last_total));
             return fail(c, SPH_ECAPACITY, "sph_read: neighbour list overflow");
         }
         const uint32_t total = off[n];
