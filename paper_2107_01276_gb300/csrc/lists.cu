@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(128) k_list_place(ListArgs a) {
 
 // Rows: only the reverse entries are placed (the coarser entries of each
 // row).  A thread per particle; most rows have none.  4.2M graded strip:
-// walk to sorted lists but for the walk itself 1.16 -> 0.57 ms, where
+// walk to sorted lists but for the walk itself 1.16 -> 0.51 ms, where
 // k_list_place copied every row into the lists; and the passes, which read
 // 32 separate lists a warp before, 1.155 -> 0.935 ms (B) and 0.935 -> 0.92
 // ms (A).
@@ -276,11 +276,20 @@ __global__ void __launch_bounds__(256) k_list_place_rev(ListArgs a) {
     if (i < (uint32_t)a.n) {
         const uint32_t r = a.rlen[i], e = r & 0xffffu;
         const uint32_t *row = a.stage + (size_t)(i >> 5) * (32 * a.stage_w) + (i & 31);
-        for (uint32_t k = r >> 16; k < e; ++k) {
-            const uint32_t j = row[32 * k];
-            if (!SPH_DCHECK(j < (uint32_t)a.n)) continue;
-            const uint32_t rp = a.off[j] + a.own[j] + atomicAdd(&a.rev[j], 1u);
-            if (rp < a.cap) a.list[rp] = i;
+        // four entries' chains of loads at once
+        for (uint32_t k = r >> 16; k < e; k += 4) {
+            uint32_t j[4], rp[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) j[u] = k + u < e ? row[32 * (k + u)] : 0xffffffffu;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                rp[u] = 0xffffffffu;
+                if (k + u < e && SPH_DCHECK(j[u] < (uint32_t)a.n))
+                    rp[u] = a.off[j[u]] + a.own[j[u]] + atomicAdd(&a.rev[j[u]], 1u);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (rp[u] < a.cap) a.list[rp[u]] = i;
         }
         if (i == (uint32_t)a.n - 1 && a.off[a.n] > a.cap) atomicOr(a.overflow, 1);
     }
@@ -348,6 +357,11 @@ __global__ void __launch_bounds__(128) k_list_fill_queue(ListArgs a) {
 // of small periodic boxes) each pair is wrapped explicitly.
 constexpr int TILE_CAP = 256;   // staged candidates per warp and batch
 constexpr int TILE_LD = 2;      // candidate loads in flight per lane
+// warps per block: two where a warp takes whole cells, whose work is uneven
+// (a block's places are free again when its last warp ends: 1, 2, 4 warps
+// 1.81, 1.65, 1.75 ms at 4.2M on the graded strip), four with teams
+template <int T>
+constexpr int TILE_WARPS = T == 1 ? 2 : 4;
 
 // The grid's levels in shared memory, a lane per level in the walk's set-up.
 struct LevTab {
@@ -764,14 +778,16 @@ __device__ __forceinline__ void tile_chunk(const ListArgs &a, const LevTab &tab,
 #define SPH_TILE_MERGE_BLOCKS 6
 #endif
 template <int T, bool MERGE = false, bool ROWS = false>
-__global__ void __launch_bounds__(128, MERGE ? SPH_TILE_MERGE_BLOCKS : (T == 1 ? 7 : 6))
+__global__ void __launch_bounds__(32 * TILE_WARPS<T>,
+                                  (MERGE ? SPH_TILE_MERGE_BLOCKS : (T == 1 ? 7 : 6)) * 4 /
+                                      TILE_WARPS<T>)
     k_list_tile(ListArgs a) {
-    __shared__ float4 sbuf[4][TILE_CAP];
-    __shared__ int spcs[4][TILE_PCS];
+    __shared__ float4 sbuf[TILE_WARPS<T>][TILE_CAP];
+    __shared__ int spcs[TILE_WARPS<T>][TILE_PCS];
     __shared__ LevTab tab;
     tab.load(a.g);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const uint32_t gw = blockIdx.x * 4u + (uint32_t)w;
+    const uint32_t gw = blockIdx.x * (uint32_t)TILE_WARPS<T> + (uint32_t)w;
     const uint32_t n = (uint32_t)a.n;
     if constexpr (T == 1) {
         const uint32_t base = gw * 32u;
@@ -1137,12 +1153,12 @@ void launch_list_walk(cudaStream_t s, const ListArgs &a, int *launches) {
     if (n <= 0) return;
     const int kind = walk_kind(a);
     if (kind == 3) {
-        k_list_tile<1><<<nblk(n, 128), 128, 0, s>>>(a);
+        k_list_tile<1><<<nblk(n, 64), 64, 0, s>>>(a);
     } else if (kind == 4) {
         if (a.rows)
-            k_list_tile<1, true, true><<<nblk(n, 128), 128, 0, s>>>(a);
+            k_list_tile<1, true, true><<<nblk(n, 64), 64, 0, s>>>(a);
         else
-            k_list_tile<1, true><<<nblk(n, 128), 128, 0, s>>>(a);
+            k_list_tile<1, true><<<nblk(n, 64), 64, 0, s>>>(a);
     } else if (kind == 2) {
         k_list_tile<4><<<nblk(n, 32), 128, 0, s>>>(a);
     } else {
