@@ -15,10 +15,10 @@ namespace sph {
 
 // List entries whose neighbour records a mixed-path pass loads together (the
 // next ones' indices are on their way meanwhile).  One lane a particle:
-// measured at 4.2M on the 1:250 strip at seven resident blocks, pass A 2, 3,
-// 4 entries 0.99, 0.92, 0.93 ms, pass B 1, 2, 3 entries (eight, seven, five
-// blocks) 1.42, 0.93, 1.04 ms.  Teams have few iterations: 26k particles,
-// pass A 2, 3 entries 16.5, 19.8 us, pass B 1, 2 entries 19.0, 20.4 us.
+// measured at 4.2M on the 1:250 strip, pass A 2, 3, 4 entries 0.99, 0.92,
+// 0.93 ms, pass B (its records still two accesses) 1, 2, 3 entries 1.42,
+// 0.93, 1.04 ms.  Teams have few iterations: 26k particles, pass A 2, 3
+// entries 16.5, 19.8 us, pass B 1, 2 entries 19.0, 20.4 us.
 template <int T>
 constexpr int UNROLL_A = T == 1 ? 3 : 2;
 template <int T>
@@ -192,8 +192,12 @@ struct PassALane {
         typename V4<R>::T A, B;
         A.x = mi; A.y = V; A.z = rho; A.w = rb2;
         B.x = a.u[i]; B.y = a.v[i]; B.z = a.p[i]; B.w = hinv;
-        a.nbA[i] = A;
-        a.nbB[i] = B;
+        if constexpr (sizeof(R) == 4) {
+            store8(a.nbA + 2 * (size_t)i, A, B);
+        } else {
+            a.nbA[i] = A;
+            a.nbB[i] = B;
+        }
     }
 };
 
@@ -230,7 +234,11 @@ struct PassBLane {
         const R beta_i = a.beta[i];
         div = diff = fax = fay = vx = vy = R(0);
         if (beta_i == R(0)) return false;
-        const typename V4<R>::T Bi = a.nbB[i];
+        typename V4<R>::T Bi;
+        if constexpr (sizeof(R) == 4)
+            Bi = a.nbA[2 * (size_t)i + 1];
+        else
+            Bi = a.nbB[i];
         hinv = Bi.w;
         dsig_i = L64 ? hinv * hinv * hinv : sigma_norm<R>() * hinv * hinv * hinv;
         rho_i = a.rho[i];
@@ -545,8 +553,7 @@ __device__ __forceinline__ void pass_b_list(const PassBArgs<R> &a, int i,
                 // an index out of range (debug builds) reads i instead
                 if (!SPH_DCHECK((unsigned)jj[u] < (unsigned)a.n)) jj[u] = i;
                 pp[u] = __ldg(&a.pk[jj[u]]);
-                AA[u] = a.nbA[jj[u]];
-                BB[u] = a.nbB[jj[u]];
+                load8(a.nbA + 2 * (size_t)jj[u], AA[u], BB[u]);
             }
 #pragma unroll
             for (int u = 0; u < U; ++u) jn[u] = E.at(k + (U + u) * T, i);
@@ -557,7 +564,9 @@ __device__ __forceinline__ void pass_b_list(const PassBArgs<R> &a, int i,
         for (int u = 0; u < U - 1; ++u) {
             if (k + u * T >= E.cnt) break;
             if (!SPH_DCHECK((unsigned)jn[u] < (unsigned)a.n)) jn[u] = i;
-            body(jn[u], __ldg(&a.pk[jn[u]]), a.nbA[jn[u]], a.nbB[jn[u]]);
+            float4 A, B;
+            load8(a.nbA + 2 * (size_t)jn[u], A, B);
+            body(jn[u], __ldg(&a.pk[jn[u]]), A, B);
         }
         if constexpr (LEAN) L.take(S);
     } else {

@@ -27,7 +27,7 @@ struct PassAArgs {
     R *rho, *beta, *pavg, *drx, *dry, *V, *rb2;
     int *nnb;
     // per-particle records for pass B: {m, V, rho, 1/(rho^2 beta)} and
-    // {u, v, p, 1/h}
+    // {u, v, p, 1/h}; FP32: both in nbA, side by side
     typename V4<R>::T *nbA, *nbB;
     int filter;                // 1: lists with a skin, test membership
 };
