@@ -384,10 +384,10 @@ __global__ void k_min_h(int n, const double *__restrict__ h,
 
 // Eq. timestep: dt = min(0.25 h_min/(U + c_s), 0.125 h_min^2/nu) into
 // dt[0], 1 / dt into dt[1].
-__device__ __forceinline__ void k_dt_body(const unsigned long long *hmin_bits,
+__device__ __forceinline__ void k_dt_body(unsigned long long hmin_bits,
                                           double U, double cs, double nu,
                                           double *dt, double *tacc, int nsteps) {
-    const double hmin = __longlong_as_double((long long)*hmin_bits);
+    const double hmin = __longlong_as_double((long long)hmin_bits);
     double v = __dmul_rn(0.25, __ddiv_rn(hmin, __dadd_rn(U, cs)));
     if (nu > 0.0) {
         double w = __dmul_rn(0.125, __ddiv_rn(__dmul_rn(hmin, hmin), nu));
@@ -404,7 +404,7 @@ __device__ __forceinline__ void k_dt_body(const unsigned long long *hmin_bits,
 
 __global__ void k_dt(const unsigned long long *hmin_bits, double U, double cs,
                      double nu, double *dt, double *tacc, int nsteps) {
-    k_dt_body(hmin_bits, U, cs, nu, dt, tacc, nsteps);
+    k_dt_body(*hmin_bits, U, cs, nu, dt, tacc, nsteps);
 }
 
 // ---------------------------------------------------------- small utils --
@@ -665,29 +665,42 @@ void launch_nbr_ids(cudaStream_t s, int n, const uint32_t *off,
                     const uint32_t *list, const int64_t *id, int64_t *out) {
     if (n > 0) k_nbr_ids<<<nblk(n, 128), 128, 0, s>>>(n, off, list, id, out);
 }
-// One block: h_min and the time step together (small sets).
+// One block: h_min and the time step together (small sets).  Bound by the
+// latency of its loads: eight of a thread are in flight at once.
+__device__ __forceinline__ unsigned long long warp_min64(unsigned long long m) {
+    for (int o = 16; o; o >>= 1) {
+        const unsigned long long t = __shfl_xor_sync(0xffffffffu, m, o);
+        m = t < m ? t : m;
+    }
+    return m;
+}
 __device__ __forceinline__ void dt_small_at(int n, const double *__restrict__ h, double U,
                                             double cs, double nu,
                                             unsigned long long *hmin_bits, double *dt,
                                             double *tacc, int nsteps) {
     __shared__ unsigned long long wm[32];
+    const unsigned long long *hb = (const unsigned long long *)h;
     unsigned long long m = ~0ull;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const unsigned long long b = (unsigned long long)__double_as_longlong(h[i]);
-        m = b < m ? b : m;
+    for (int i0 = threadIdx.x; i0 < n; i0 += 8 * blockDim.x) {
+        unsigned long long b[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int i = i0 + k * (int)blockDim.x;
+            b[k] = i < n ? __ldg(&hb[i]) : ~0ull;
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) m = b[k] < m ? b[k] : m;
     }
-    for (int o = 16; o; o >>= 1) {
-        const unsigned long long t = __shfl_xor_sync(0xffffffffu, m, o);
-        m = t < m ? t : m;
-    }
+    m = warp_min64(m);
     if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = m;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = wm[w] < m ? wm[w] : m;
-        *hmin_bits = m;
+    if (threadIdx.x < 32) {
+        m = warp_min64(threadIdx.x < (blockDim.x >> 5) ? wm[threadIdx.x] : ~0ull);
+        if (threadIdx.x == 0) {
+            *hmin_bits = m;
+            k_dt_body(m, U, cs, nu, dt, tacc, nsteps);
+        }
     }
-    __syncthreads();
-    if (threadIdx.x == 0) k_dt_body(hmin_bits, U, cs, nu, dt, tacc, nsteps);
 }
 
 __global__ void __launch_bounds__(1024)
