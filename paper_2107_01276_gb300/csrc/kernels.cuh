@@ -176,14 +176,18 @@ __device__ __forceinline__ float frcp_ftz(float b) {
 constexpr float F32_LEAST = 1.17549435e-38f;   // least normal
 
 // The bases of the clipped quintic (qs_w above) at two q = r / h each, nh =
-// {-1 / h, -1 / h'}: one FMA a base, the product with r not rounded apart.
+// {-1 / h, -1 / h'}.  3 - q is rounded once and 2 - q and 1 - q follow from it
+// exactly, so the rounding acts like one error of q, which mostly cancels in
+// the derivative.  (Each base by its own FMA made the momentum rates of the
+// 1:250 strip 6 % less accurate, all three from a rounded q pass B 5 %
+// slower.)
 struct Qs2 {
     F2 a, b, c;
     __device__ __forceinline__ Qs2(float r, F2 nh) {
-        const F2 rr = f2(r);
-        a = clip2(fma2(rr, nh, f2(3.0f)));
-        b = clip2(fma2(rr, nh, f2(2.0f)));
-        c = clip2(fma2(rr, nh, f2(1.0f)));
+        const F2 t = fma2(f2(r), nh, f2(3.0f));
+        a = clip2(t);
+        b = clip2(add2(t, f2(-1.0f)));
+        c = clip2(add2(t, f2(-2.0f)));
     }
     // s = -(dw/dq) / 5
     __device__ __forceinline__ F2 s() const {
@@ -192,10 +196,9 @@ struct Qs2 {
     }
     __device__ __forceinline__ void ws(F2 &w, F2 &s) const {
         const F2 a2 = mul2(a, a), b2 = mul2(b, b), c2 = mul2(c, c);
-        const F2 a4 = mul2(a2, a2), b4 = mul2(mul2(b2, f2(-6.0f)), b2),
-                 c4 = mul2(mul2(c2, f2(15.0f)), c2);
-        s = add2(a4, add2(b4, c4));
-        w = fma2(a4, a, fma2(b4, b, mul2(c4, c)));
+        const F2 b6 = mul2(b2, f2(-6.0f)), c4 = mul2(mul2(c2, f2(15.0f)), c2);
+        s = fma2(a2, a2, fma2(b6, b2, c4));
+        w = fma2(mul2(a2, a2), a, fma2(mul2(b6, b2), b, mul2(c4, c)));
     }
 };
 
@@ -227,7 +230,7 @@ template <> struct V4<double> { using T = double4_32a; };
 
 // The FP32 pass-B record of a neighbour, its two halves side by side: one
 // 32-byte access (pass B is bound by the L1 data pipe of its gathers; two
-// 16-byte ones took 0.935 instead of 0.89 ms at 4.2M on the graded strip).
+// 16-byte ones took 5 % longer at 4.2M on the graded strip).
 __device__ __forceinline__ void load8(const float4 *p, float4 &a, float4 &b) {
     asm("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
         : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)

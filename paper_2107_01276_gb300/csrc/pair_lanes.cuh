@@ -153,6 +153,8 @@ struct PassALane {
         ay = team_sum<T>(tm.mask, ay);
         cnt = team_sum<T>(tm.mask, cnt);
         if (tm.lane != 0) return;
+        // mixed: sigma / h^2 cancels in beta
+        [[maybe_unused]] const R beta_lean = R(2.5) * (hinv * srw) / rho;
         if constexpr (LEAN) {
             srw *= R(-5);
             ax *= R(-40) * sigma_norm<R>();
@@ -160,7 +162,7 @@ struct PassALane {
         }
         const R sig = sigma_norm<R>() * hinv * hinv;
         rho *= sig;
-        const R beta = -(sig * hinv * srw) / (rho * R(2));
+        const R beta = LEAN && !L64 ? beta_lean : -(sig * hinv * srw) / (rho * R(2));
         R drx = R(0), dry = R(0);
         if (beta != R(0)) {
             const R c = R(-0.5) * hi * hi / (R)a.rho0;

@@ -20,12 +20,12 @@
 namespace sph {
 
 // resident 128-thread blocks per SM the mixed one-lane passes are compiled
-// for (72 and 80 registers, measured at 4.2M on the graded strip: pass A at
-// seven and eight blocks 0.92 and 1.05 ms, pass B at five, six, seven 0.92,
-// 0.89, 1.53 ms; with too few registers the loads of an iteration are no
-// longer in flight together)
+// for (measured at 4.2M on the graded strip: pass A at seven and eight
+// blocks 0.92 and 1.05 ms, pass B at five, six, seven 0.92, 0.93, 1.52 ms;
+// with too few registers the loads of an iteration are no longer in flight
+// together)
 constexpr int PASS_A_BLOCKS = 7;
-constexpr int PASS_B_BLOCKS = 6;
+constexpr int PASS_B_BLOCKS = 5;
 // Team forms (T > 1: small and walled sets) and the batched forms keep six
 // and five blocks (80 / 96 registers), for their wall loops.
 template <typename R, int T>
