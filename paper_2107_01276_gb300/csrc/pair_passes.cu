@@ -36,9 +36,8 @@ constexpr int pass_blocks(int lane1) {
 // ---------------------------------------------------------------- pass A --
 // Pass A of particle i over its list (arithmetic in PassALane): a team of T
 // threads shares particle i.  WALLS = false: a set without wall particles,
-// compiled without the wall loop (whose registers made the one-lane pass B
-// spill at the eight-block bound) and, on the FP64 path, with the LEAN
-// arithmetic (kernels.cuh).
+// compiled without the wall loop (and its
+// registers) and with the LEAN arithmetic (kernels.cuh).
 template <typename R, int T, bool WALLS>
 __device__ __forceinline__ void pass_a_at(const PassAArgs<R> &a, int i,
                                           const Team<T> &tm) {
