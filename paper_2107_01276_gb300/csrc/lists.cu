@@ -906,12 +906,18 @@ __device__ __forceinline__ void sort_regs(uint32_t *seg, uint32_t len) {
         if (t < (int)len) seg[t] = r[t];
 }
 
-__device__ __forceinline__ void list_sort_rev_at(int i, int n, const uint32_t *off,
+// Also the last word on an overflowed build: its offsets are cut to the
+// capacity, so what reads the lists before the overflow is reported meets the
+// entries that were written and never leaves the buffer.  (A neighbour's
+// thread may see an offset raw or cut: past the capacity either way.)
+__device__ __forceinline__ void list_sort_rev_at(int i, int n, uint32_t *off,
                                                  const uint32_t *own, uint32_t *list,
                                                  uint32_t cap, uint32_t *longq,
                                                  uint32_t *nlong) {
     if (i >= n) return;
-    const uint32_t b = off[i] + (own ? own[i] : 0u), e = off[i + 1];
+    const uint32_t o = off[i], b = o + (own ? own[i] : 0u), e = off[i + 1];
+    if (o > cap) off[i] = cap;
+    if (i == n - 1 && e > cap) off[n] = cap;
     if (e > cap || e <= b + 1) return;
     const uint32_t len = e - b;
     if (len > SORT_REG) {
@@ -927,7 +933,7 @@ __device__ __forceinline__ void list_sort_rev_at(int i, int n, const uint32_t *o
         sort_regs<SORT_REG>(list + b, len);
 }
 
-__global__ void k_list_sort_rev(int n, const uint32_t *off, const uint32_t *own,
+__global__ void k_list_sort_rev(int n, uint32_t *off, const uint32_t *own,
                                 uint32_t *list, uint32_t cap, uint32_t *longq,
                                 uint32_t *nlong) {
     list_sort_rev_at(blockIdx.x * blockDim.x + threadIdx.x, n, off, own, list, cap, longq,
@@ -1044,7 +1050,7 @@ __global__ void __launch_bounds__(128) k_list_sort_long_batch(const SortSegRec *
 // ------------------------------------------------------------- launchers --
 static inline int nblk_s(int n, int bs) { return (n + bs - 1) / bs; }
 
-void sort_segments(cudaStream_t s, int n, const uint32_t *off, uint32_t *list,
+void sort_segments(cudaStream_t s, int n, uint32_t *off, uint32_t *list,
                    uint32_t cap, uint32_t *longq, uint32_t *nlong,
                    int *launches) {
     if (n <= 0) return;

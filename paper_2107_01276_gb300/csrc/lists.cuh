@@ -97,7 +97,8 @@ int pack_batch_blocks_per_sm();
 // change no result).
 struct SortSegRec {
     int n;
-    const uint32_t *off, *own;
+    uint32_t *off;
+    const uint32_t *own;
     uint32_t *list;
     uint32_t cap;
     uint32_t *longq, *nlong;
@@ -117,7 +118,8 @@ void launch_anchor_pack(cudaStream_t s, int n, const double *x,
                         const double *A, const Anchor &an, float4 *pk);
 // The walk (own entries staged, reverse entries counted), then the
 // offsets (off has n + 1 entries), then the fill;
-// entries past a.cap are dropped and flag a.overflow.  Before the walk,
+// entries past a.cap are dropped and flag a.overflow, and the offsets end at
+// a.cap (list_sort_rev_at).  Before the walk,
 // rev[0..n) and the counters nqueue, max_own and nlong must be zero (the
 // rebuild's reset and key kernels do that).
 void launch_list_walk(cudaStream_t s, const ListArgs &a, int *launches);
@@ -128,8 +130,8 @@ void build_lists_fill(cudaStream_t s, ListArgs a, bool mixed, bool queue,
                       int *launches);
 // Each segment [off[i], off[i+1]) of list in ascending order (short ones in
 // registers, long ones queued in longq / *nlong, which must be zero, for a
-// warp sort).
-void sort_segments(cudaStream_t s, int n, const uint32_t *off, uint32_t *list,
+// warp sort); offsets past cap cut to it.
+void sort_segments(cudaStream_t s, int n, uint32_t *off, uint32_t *list,
                    uint32_t cap, uint32_t *longq, uint32_t *nlong,
                    int *launches);
 

@@ -992,16 +992,17 @@ sph_status check_overflow(sph_ctx *c, const char *who) {
     cudaMemcpyAsync(&flags[0], c->d_overflow, sizeof(int), cudaMemcpyDeviceToHost, c->s);
     cudaMemcpyAsync(&flags[1], c->d_skin_err, sizeof(int), cudaMemcpyDeviceToHost, c->s);
     if (cudaStreamSynchronize(c->s) != cudaSuccess) return cuda_check(c, who);
-    if (flags[1]) {
-        cudaMemsetAsync(c->d_skin_err, 0, sizeof(int), c->s);
+    if (flags[1]) cudaMemsetAsync(c->d_skin_err, 0, sizeof(int), c->s);
+    if (flags[0]) {   // first: a step on cut lists may also throw particles far
+        cudaMemsetAsync(c->d_overflow, 0, sizeof(int), c->s);
+        memset(c->last_total, 0, sizeof(c->last_total));   // next builds size exactly
+        return fail(c, SPH_ECAPACITY, std::string(who) + ": neighbour list overflow");
+    }
+    if (flags[1])
         return fail(c, SPH_ENONFINITE,
                     std::string(who) + ": particles moved farther than the neighbour-list "
                     "skin within one step (flow speed far above U_ref + cs)");
-    }
-    if (!flags[0]) return SPH_OK;
-    cudaMemsetAsync(c->d_overflow, 0, sizeof(int), c->s);
-    memset(c->last_total, 0, sizeof(c->last_total));   // next builds size exactly
-    return fail(c, SPH_ECAPACITY, std::string(who) + ": neighbour list overflow");
+    return SPH_OK;
 }
 
 // ================================================================ C ABI ==
@@ -1198,10 +1199,11 @@ sph_status sph_load_particles(sph_ctx *c, sph_kind kind, long long n,
     std::swap(c->id, c->id_alt);
     c->n = (int)n;
     c->next_id = n > 0 && src->id ? chk.idmax + 1 : n;
-    // a new state: a non-finite rate or skin overrun reported for the old
-    // one no longer applies
+    // a new state: a non-finite rate, skin overrun or list overflow of the
+    // old one no longer applies
     cudaMemsetAsync(c->d_nonfinite, 0, sizeof(int), c->s);
     cudaMemsetAsync(c->d_skin_err, 0, sizeof(int), c->s);
+    cudaMemsetAsync(c->d_overflow, 0, sizeof(int), c->s);
     cudaStreamSynchronize(c->s);
     c->grid_valid = c->rhs_valid = c->have_dt = false;
     return cuda_check(c, "sph_load_particles");
@@ -1385,8 +1387,9 @@ static sph_status read_field(sph_ctx *c, sph_field field, void *dst, long long c
     case SPH_F_BETA: case SPH_F_PAVG: case SPH_F_DRX: case SPH_F_DRY:
     case SPH_F_DPDT: case SPH_F_DUDT: case SPH_F_DVDT: {
         if (!c->rhs_valid) return fail(c, SPH_ESTATE, "sph_read: no right-hand side at this state");
-        if ((st = check_overflow(c, "sph_read")) != SPH_OK) return st;
+        // (a call that asks for the size must not use up the report)
         if ((st = need(n)) != SPH_OK) return st;
+        if ((st = check_overflow(c, "sph_read")) != SPH_OK) return st;
         const void *srcs[] = {c->beta, c->pavg, c->drx, c->dry, c->dpdt, c->dudt, c->dvdt};
         return read_R(c, srcs[field - SPH_F_BETA], (double *)dst, n);
     }

@@ -79,7 +79,7 @@ struct WallListArgs {
     float reach;
     uint32_t *cnt;                // n + 1 counts (zeroed by the build's key
                                   // and reset kernels)
-    const uint32_t *off;          // n + 1 offsets (fill pass)
+    uint32_t *off;                // n + 1 offsets (fill pass; cut to cap)
     uint32_t *cur;                // n cursors (zeroed likewise)
     uint32_t *list;
     uint32_t cap;
