@@ -179,6 +179,12 @@ struct sph_ctx {
     float skin = 1.0f;          // skin factor of the current lists (1: exact)
     int *d_skin_err = nullptr;  // set when particles outran the skin
     int last_total_n[3] = {};
+    // with rows: entries that were in them at the last such read-back
+    unsigned long long last_rows = 0, *d_rows = nullptr;
+    // fluid sets loaded so far; the last one's count and least and largest h
+    int loads = 0;
+    long long load_n = -1;
+    double load_h[2] = {};
     long long steps = 0;
     int launches = 0;
     bool timing = false;
@@ -225,11 +231,16 @@ bool want_wall_lists(const sph_ctx *c);
 sph_status rebuild(sph_ctx *c, bool mid_step, bool exact = true,
                           float skin = 1.0f, bool for_walls = true, bool rows = false);
 // The list forms whose sizes are remembered apart: exact, with a skin, with
-// a skin and rows.  A build of a form needs no read-back when the last total
-// read back was at most half the list buffer, at a particle count within
+// a skin and rows.  A build of a form needs no read-back when list_need of
+// the last one is at most half the list buffer, at a particle count within
 // 10 %.
 enum ListForm { LIST_EXACT, LIST_SKIN, LIST_ROWS };
 ListForm step_form(sph_ctx *c);          // of a step's first build
+// Entries of the last build of a form that read its size back.  With rows a
+// list holds the reverse entries and the own entries of particles whose rows
+// overflow: none of most sets, all of a denser one loaded after it, so a
+// context loaded more than once counts the entries in the rows too.
+size_t list_need(const sph_ctx *c, ListForm f);
 bool list_sized(const sph_ctx *c, ListForm f);
 WallBcArgs wall_bc_args(sph_ctx *c);
 void run_passes(sph_ctx *c);

@@ -295,6 +295,16 @@ __global__ void __launch_bounds__(256) k_list_place_rev(ListArgs a) {
     }
 }
 
+// Only builds that read their size back sum the rows.
+__global__ void __launch_bounds__(256)
+    k_row_total(int n, const uint32_t *__restrict__ rlen, unsigned long long *total) {
+    unsigned long long t = 0;
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256)
+        t += rlen[i] & 0xffffu;
+    for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((threadIdx.x & 31) == 0) atomicAdd(total, t);
+}
+
 // Second walk for the queued particles (more than stage_w own entries):
 // same order as k_list_gather; teams take queue entries in turn.
 template <int T>
@@ -1183,6 +1193,14 @@ void list_offsets(cudaStream_t s, const ListArgs &a, SortScratch &sc, int *launc
         return;
     }
     scan_list_offsets(s, a.own, a.rev, a.off, n, sc, launches);
+}
+
+void launch_row_total(cudaStream_t s, int n, const uint32_t *rlen, unsigned long long *total,
+                      int *launches) {
+    cudaMemsetAsync(total, 0, sizeof(*total), s);
+    if (n <= 0) return;
+    k_row_total<<<std::min(152 * 8, nblk(n, 256)), 256, 0, s>>>(n, rlen, total);
+    *launches += 1;
 }
 
 void build_lists_fill(cudaStream_t s, ListArgs a, bool mixed, bool queue,

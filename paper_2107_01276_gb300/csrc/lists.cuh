@@ -124,6 +124,9 @@ void launch_anchor_pack(cudaStream_t s, int n, const double *x,
 // rebuild's reset and key kernels do that).
 void launch_list_walk(cudaStream_t s, const ListArgs &a, int *launches);
 void list_offsets(cudaStream_t s, const ListArgs &a, SortScratch &sc, int *launches);
+// *total = entries in the rows (ListArgs::rlen)
+void launch_row_total(cudaStream_t s, int n, const uint32_t *rlen, unsigned long long *total,
+                      int *launches);
 // queue: launch the second walk for rows that overflowed (false when the
 // caller knows none did).
 void build_lists_fill(cudaStream_t s, ListArgs a, bool mixed, bool queue,

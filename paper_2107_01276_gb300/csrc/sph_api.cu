@@ -246,9 +246,13 @@ ListForm step_form(sph_ctx *c) {
     return list_rows_for(list_args(c)) ? LIST_ROWS : LIST_SKIN;
 }
 
+size_t list_need(const sph_ctx *c, ListForm f) {
+    return c->last_total[f] + (f == LIST_ROWS && c->loads > 1 ? (size_t)c->last_rows : 0);
+}
+
 bool list_sized(const sph_ctx *c, ListForm f) {
     const long long n = c->n, ltn = c->last_total_n[f];
-    return c->last_total[f] > 0 && (size_t)c->last_total[f] * 2 <= c->list_cap &&
+    return c->last_total[f] > 0 && list_need(c, f) * 2 <= c->list_cap &&
            n * 10 <= ltn * 11 && n * 10 >= ltn * 9;
 }
 
@@ -341,6 +345,11 @@ sph_status rebuild(sph_ctx *c, bool mid_step, bool exact,
         cudaMemcpyAsync(&max_own, c->d_max_own, sizeof(uint32_t), cudaMemcpyDeviceToHost, c->s);
         if (walls)
             cudaMemcpyAsync(&wtotal, c->woff + n, sizeof(uint32_t), cudaMemcpyDeviceToHost, c->s);
+        if (la.rows) {
+            launch_row_total(c->s, n, c->rlen, c->d_rows, &c->launches);
+            cudaMemcpyAsync(&c->last_rows, c->d_rows, sizeof(c->last_rows),
+                            cudaMemcpyDeviceToHost, c->s);
+        }
         if (cudaStreamSynchronize(c->s) != cudaSuccess) return cuda_check(c, "rebuild sync");
         if (walls && (size_t)wtotal * 2 > c->wcap) {
             const size_t want = std::min<size_t>(2 * (size_t)wtotal + 4096, 0xffffffffull);
@@ -365,8 +374,8 @@ sph_status rebuild(sph_ctx *c, bool mid_step, bool exact,
             c->stage_want = std::min<uint32_t>(256, (max_own + max_own / 4 + 15) & ~15u);
         // twice the entries found: the next builds skip this read-back
         // (and sph_step can replay its captured graph)
-        if ((size_t)total * 2 > c->list_cap) {
-            size_t want = 2 * (size_t)total + 1024;
+        if (list_need(c, form) * 2 > c->list_cap) {
+            size_t want = 2 * list_need(c, form) + 1024;
             if (want > 0xffffffffull) want = 0xffffffffull;
             if ((size_t)total > want)
                 return fail(c, SPH_ECAPACITY, "neighbour lists exceed 2^32 entries");
@@ -516,7 +525,7 @@ void free_ctx(sph_ctx *c) {
                   c->pf, c->uf, c->vf, c->nnb, c->skey, c->perm,
                   c->sc.key_alt, c->sc.val_alt, c->sc.counts, c->sc.scan_tmp,
                   c->tkey, c->tstart, c->tend, c->tmaxh, c->bbox, c->level_mask,
-                  c->d_dt, c->d_t, c->d_hmin, c->d_nonfinite,
+                  c->d_dt, c->d_t, c->d_hmin, c->d_nonfinite, c->d_rows,
                   c->d_total, c->lvl, c->pk, c->own, c->rev, c->off, c->list,
                   c->d_overflow, c->d_skin_err, c->longq, c->d_nlong, c->stage, c->rlen, c->lqueue, c->lqref, c->d_max_own,
                   c->d_nlq, c->tmp_a, c->tmp_b,
@@ -886,7 +895,7 @@ sph_status new_ctx(const sph_params *p, cudaStream_t stream, bool has_ds,
     ok = ok && dalloc(&c->bbox, MAX_LEVELS * 4, c->s) && dalloc(&c->level_mask, 1, c->s);
     ok = ok && dalloc(&c->d_dt, 2, c->s) && dalloc(&c->d_t, 1, c->s) && dalloc(&c->d_hmin, 1, c->s) &&
          dalloc(&c->d_nonfinite, 1, c->s) && dalloc(&c->d_total, 1, c->s) &&
-         dalloc(&c->d_skin_err, 1, c->s) &&
+         dalloc(&c->d_rows, 1, c->s) && dalloc(&c->d_skin_err, 1, c->s) &&
          dalloc(&c->d_overflow, 1, c->s);
     ok = ok && dalloc(&c->lvl, N, c->s) && dalloc(&c->pk, N, c->s) && dalloc(&c->own, N, c->s) &&
          dalloc(&c->rev, N, c->s) && dalloc(&c->off, N + 1, c->s) &&
@@ -1199,6 +1208,13 @@ sph_status sph_load_particles(sph_ctx *c, sph_kind kind, long long n,
     std::swap(c->id, c->id_alt);
     c->n = (int)n;
     c->next_id = n > 0 && src->id ? chk.idmax + 1 : n;
+    // another kind of set: the sizes of the old one's lists say nothing
+    if (n != c->load_n || hmin != c->load_h[0] || hmax != c->load_h[1])
+        memset(c->last_total, 0, sizeof(c->last_total));
+    c->loads += 1;
+    c->load_n = n;
+    c->load_h[0] = hmin;
+    c->load_h[1] = hmax;
     // a new state: a non-finite rate, skin overrun or list overflow of the
     // old one no longer applies
     cudaMemsetAsync(c->d_nonfinite, 0, sizeof(int), c->s);

@@ -5,7 +5,7 @@ import pytest
 
 from paper_2107_01276_gb300 import sph
 from paper_2107_01276_gb300 import workloads as wl
-from tests.helpers import by_id, cuda_ok, stream_handle
+from tests.helpers import MIXED_TOL, by_id, cuda_ok, stream_handle
 
 pytestmark = pytest.mark.gpu
 STATE = ["x", "y", "u", "v", "p", "rho"]
@@ -81,3 +81,35 @@ def test_overflow_without_readback_is_reported_and_left_behind(case, precision, 
     ref.close()
     for f in STATE:
         assert np.array_equal(a[f], b[f]), f
+
+
+@pytest.mark.parametrize("second", ["coarser_h", "denser", "fewer"])
+def test_reloaded_context_takes_a_set_whose_rows_overflow(second):
+    """A set whose step keeps every own entry in the rows, then one of the
+    same count with more own entries a particle than a row holds: with
+    larger h, or denser by 1.6 at the same h, or with a tenth fewer
+    particles and larger h.  The steps after the second load are a fresh
+    context's to the mixed tolerance of the change, once a step."""
+    d = wl.taylor_green(nx=230, hdx=1.2, jitter=0.1, seed=8)
+    pt = dict(d["particles"])
+    if second == "denser":
+        pt = _packed(pt, x=0.62)
+    else:
+        pt["h"] = pt["h"] * (1.55 / 1.2)
+        if second == "fewer":
+            pt = {k: v[:48100] for k, v in pt.items()}
+    sim = _sim(d, sph.SPH_MIXED)
+    sim.step(2)
+    sim.load(pt)
+    ref = _sim(dict(d, particles=pt), sph.SPH_MIXED)
+    out = []
+    for s in (sim, ref):
+        s.step(1)
+        one = by_id(s, STATE)
+        s.step(3)
+        out.append((one, by_id(s, STATE)))
+        s.close()
+    for a, b, k in zip(*out, (1, 4)):
+        for f in ("u", "v", "p"):
+            change = np.abs(b[f] - pt[f]).max()
+            assert np.abs(a[f] - b[f]).max() <= k * MIXED_TOL * change, f
