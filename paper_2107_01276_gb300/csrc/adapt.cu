@@ -384,7 +384,7 @@ __global__ void __launch_bounds__(128) k_density_mbar(ShiftArgs a, int want_h) {
         if (!want_h && !(r2 < R(9) * hi * hi)) continue;
         if constexpr (lean64<R, LEAN>) {
             R w, s;
-            qs_ws(nonzero(r2) ? __dmul_rn(__dmul_rn(r2, frsqrt_lean(r2)), hinv) : R(0), w, s);
+            qs_ws(is_normal(r2) ? __dmul_rn(__dmul_rn(r2, frsqrt_lean(r2)), hinv) : R(0), w, s);
             rho += in.m[j] * w;
         } else {
             rho += in.m[j] * qs_w<R>(sqrt(r2) * hinv);   // zero beyond 3 h_i
@@ -454,7 +454,7 @@ __global__ void __launch_bounds__(128) k_shift_compute(ShiftArgs a) {
         }
         R Vg;
         if constexpr (lean64<R, LEAN>) {
-            if (!nonzero(r2)) continue;
+            if (!is_normal(r2)) continue;
             const R rinv = frsqrt_lean(r2), r = __dmul_rn(r2, rinv);
             // times -40 sigma / rho0 at the end
             const R hsinv = frcp(hi + hj);

@@ -121,8 +121,13 @@ __device__ __forceinline__ void qs_ws(double q, double &w, double &s) {
     s = __fma_rn(s, p.t, p.coef(8.0, 4.0, 0.0));
     s = __fma_rn(s, p.t, p.coef(10.0, 1.0, 0.0));
 }
-// x != 0 for x >= 0, on the integer pipe
-__device__ __forceinline__ bool nonzero(double x) { return __double_as_longlong(x) != 0; }
+// Whether x >= 0 is a normal number (or infinite, or NaN), on the integer
+// pipe.  A squared separation below that (r < 1.5e-154) counts as zero: the
+// estimate above flushes it and returns infinity.  The kernels are at
+// their r = 0 values to the last bit long before.
+__device__ __forceinline__ bool is_normal(double x) {
+    return (uint32_t)__double2hiint(x) >= 0x00100000u;
+}
 
 // Mixed pair sums of sets without walls (LEAN): two values share an
 // instruction where the formulas come in pairs: the axes of a separation, u

@@ -69,7 +69,7 @@ struct PassALane {
                                          R dy, R r2) {
         if constexpr (L64) {
             // r = 0 (i itself): rinv = 0 and the shift term is zero
-            const R rinv = nonzero(r2) ? frsqrt_lean(r2) : R(0);
+            const R rinv = is_normal(r2) ? frsqrt_lean(r2) : R(0);
             const R r = __dmul_rn(r2, rinv);
             R w, s;
             qs_ws(__dmul_rn(r, hinv), w, s);
@@ -270,7 +270,7 @@ struct PassBLane {
                                          R ujy, R ugx, R ugy) {
         R gi = 0, gj = 0;
         if constexpr (L64) {
-            const R rinv = nonzero(r2) ? frsqrt_lean(r2) : R(0);
+            const R rinv = is_normal(r2) ? frsqrt_lean(r2) : R(0);
             const R r = __dmul_rn(r2, rinv);
             const R k = R(-5) * sigma_norm<R>() * rinv;
             // dsig_i: 1 / h_i^3
