@@ -268,9 +268,7 @@ static size_t batch_bytes_per_instance() {
 // one rebuild() makes without read-back, kernel for kernel.
 static bool small_build_ok(sph_ctx *c, float skin) {
     const int n = c->n;
-    if (n < 2 || !radix_small_takes(n, 2 * c->mbits + c->lbits) || n > scan_small_max() ||
-        n > dt_small_max())
-        return false;
+    if (n < 2 || n > radix_small_max() || n > scan_small_max() || n > dt_small_max()) return false;
     if (!radix_small_available() || want_wall_lists(c) || c->timing) return false;
     if (c->stage_want > c->stage_w) return false;
     if (2 * c->mbits + c->lbits <= 0) return false;
@@ -388,10 +386,10 @@ static bool launch_small_builds(sph_batch *b, Stager &st, const std::vector<Smal
     std::vector<ScanSmallRec> sc;
     std::vector<SortSegRec> seg;
     std::vector<int> i_one, i_rr, i_256, i_128, i_fq, i_sl;
-    int max_smem = 0;
+    int max_n = 0;
     for (const SmallBuild &B : bs) {
         const int n = B.c->n;
-        max_smem = std::max(max_smem, radix_small_bytes(n, B.rs.passes));
+        max_n = std::max(max_n, n);
         if (with_dt) dt.push_back(B.dt);
         rr.push_back(B.rr);
         keys.push_back(B.keys);
@@ -469,7 +467,7 @@ static bool launch_small_builds(sph_batch *b, Stager &st, const std::vector<Smal
     launch_rebuild_reset_batch(b->s, (const RebuildReset *)(st.d + grr.off_args), sp(grr));
     launch_keys_batch(b->s, (const KeysRec *)(st.d + gkeys.off_args), sp(gkeys));
     if (!launch_radix_small_batch(b->s, (const RadixSmallRec *)(st.d + grs.off_args), sp(grs),
-                                  max_smem))
+                                  max_n))
         return false;
     launch_gather_batch(b->s, (const GatherPackRec *)(st.d + ggp.off_args), sp(ggp));
     launch_pack_batch(b->s, (const PackArgs *)(st.d + gpk.off_args), sp(gpk), b->pack_blocks);

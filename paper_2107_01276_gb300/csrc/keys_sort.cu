@@ -291,30 +291,32 @@ __global__ void __launch_bounds__(RS_THREADS)
 // with __match_any_sync against per-(warp, digit) counts, scans the counts
 // digit-major (a warp takes 8 digits, a lane a warp's count), scatters keys
 // and positions into shared memory and reloads them in the new order, so
-// the sort is stable exactly like the tiled form and global memory sees one
-// read and one write.  Keys of at most 32 bits travel as such; wider ones
-// take half the items.  Bound by the latency of its chain of passes: 5 us
-// at 2.5k particles and 3 digits, 9.5 us at 16k (the former form, with two
-// rankings a pass and passes through global memory, took 10 and 29).
+// the sort is stable exactly like the tiled form.  A key travels as 32 bits:
+// its low word through the first four passes; a wider key's high word is
+// then fetched from its place in the input, and the whole key at the end
+// (64-bit keys in registers left room for half the items, and wide sets of
+// 8193 to 16384 particles to the tiled sort's fifteen launches or more).
+// Bound by the latency of its chain of passes: 5 us at 2.5k particles and 3
+// digits, 9.5 us at 16k (the former form, with two rankings a pass and
+// passes through global memory, took 10 and 29).
 constexpr int RSS_THREADS = 1024;
 constexpr int RSS_WARPS = RSS_THREADS / 32;
 constexpr int RSS_MAX = 16384;
-constexpr int RSS_MAX64 = RSS_MAX / 2;     // keys wider than 32 bits
 
-static size_t radix_small_smem(int n, int passes) { return (size_t)n * (passes <= 4 ? 6 : 10); }
+static size_t radix_small_smem(int n) { return (size_t)n * 6; }
 
-template <typename K, int IT>
+template <int IT>
 __device__ __forceinline__ void radix_small_body(int n, int passes, uint64_t *ka,
                                                  uint32_t *va, uint32_t (*cnt)[257],
                                                  uint32_t *dtot) {
-    extern __shared__ uint64_t rss_buf[];          // n keys, then n positions
-    K *sk = (K *)rss_buf;
+    extern __shared__ uint64_t rss_buf[];          // n key words, then n positions
+    uint32_t *sk = (uint32_t *)rss_buf;
     uint16_t *si = (uint16_t *)(sk + n);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const int rows = (n + RSS_THREADS - 1) / RSS_THREADS;   // items a lane, <= IT
     const int wb = w * rows * 32 + lane;
-    K key[IT];
+    uint32_t key[IT];
     uint32_t ir[IT];                               // position | rank << 16
 #pragma unroll
     for (int s = 0; s < IT; ++s) {
@@ -322,12 +324,17 @@ __device__ __forceinline__ void radix_small_body(int n, int passes, uint64_t *ka
         key[s] = 0;
         ir[s] = 0;
         if (s < rows && e < n) {
-            key[s] = (K)ka[e];
+            key[s] = (uint32_t)ka[e];
             ir[s] = (uint32_t)e;
         }
     }
     for (int p = 0; p < passes; ++p) {
-        const int shift = 8 * p;
+        const int shift = 8 * (p & 3);
+        if (p == 4) {
+#pragma unroll
+            for (int s = 0; s < IT; ++s)
+                if (s < rows && wb + s * 32 < n) key[s] = (uint32_t)(ka[ir[s]] >> 32);
+        }
         for (int t = threadIdx.x; t < RSS_WARPS * 257; t += RSS_THREADS) (&cnt[0][0])[t] = 0;
         __syncthreads();
 #pragma unroll
@@ -398,48 +405,52 @@ __device__ __forceinline__ void radix_small_body(int n, int passes, uint64_t *ka
             }
         }
     }
-    // the values of the final order, all read before any is replaced
+    // the keys and values of the final order, all read before any is replaced
+    if (passes > 4) {   // (the low words wait in shared memory)
+#pragma unroll
+        for (int s = 0; s < IT; ++s)
+            if (s < rows && wb + s * 32 < n) sk[wb + s * 32] = (uint32_t)ka[ir[s]];
+        __syncthreads();
+#pragma unroll
+        for (int s = 0; s < IT; ++s)
+            if (s < rows && wb + s * 32 < n)
+                ka[wb + s * 32] = ((uint64_t)key[s] << 32) | sk[wb + s * 32];
+    } else {
+#pragma unroll
+        for (int s = 0; s < IT; ++s)
+            if (s < rows && wb + s * 32 < n) ka[wb + s * 32] = key[s];
+    }
 #pragma unroll
     for (int s = 0; s < IT; ++s)
         if (s < rows && wb + s * 32 < n) ir[s] = va[ir[s]];
     __syncthreads();
 #pragma unroll
-    for (int s = 0; s < IT; ++s) {
-        const int e = wb + s * 32;
-        if (s < rows && e < n) {
-            ka[e] = key[s];
-            va[e] = ir[s];
-        }
-    }
+    for (int s = 0; s < IT; ++s)
+        if (s < rows && wb + s * 32 < n) va[wb + s * 32] = ir[s];
 }
 
 __device__ __forceinline__ void radix_small_at(int n, int passes, uint64_t *ka, uint32_t *va) {
     __shared__ uint32_t cnt[RSS_WARPS][257];       // padded: a lane a row is conflict-free
     __shared__ uint32_t dtot[256];
-    if (passes <= 4)
-        radix_small_body<uint32_t, RSS_MAX / RSS_THREADS>(n, passes, ka, va, cnt, dtot);
-    else
-        radix_small_body<uint64_t, RSS_MAX64 / RSS_THREADS>(n, passes, ka, va, cnt, dtot);
+    radix_small_body<RSS_MAX / RSS_THREADS>(n, passes, ka, va, cnt, dtot);
 }
 
 // Alone, the sort is compiled for the items a lane really has: the unrolled
 // 16 of the largest sets are many times the instructions that a set of a
 // thousand needs, and their fetching was most of its time.
-template <typename K, int IT>
+template <int IT>
 __global__ void __launch_bounds__(RSS_THREADS)
     k_radix_small(int n, int passes, uint64_t *ka, uint32_t *va) {
     __shared__ uint32_t cnt[RSS_WARPS][257];
     __shared__ uint32_t dtot[256];
-    radix_small_body<K, IT>(n, passes, ka, va, cnt, dtot);
+    radix_small_body<IT>(n, passes, ka, va, cnt, dtot);
 }
 using RadixSmallFn = void (*)(int, int, uint64_t *, uint32_t *);
-static RadixSmallFn radix_small_fn(int n, int passes) {
-    if (passes <= 4)
-        return n <= RSS_THREADS ? k_radix_small<uint32_t, 1>
-               : n <= 4 * RSS_THREADS ? k_radix_small<uint32_t, 4>
-                                      : k_radix_small<uint32_t, RSS_MAX / RSS_THREADS>;
-    return n <= RSS_THREADS ? k_radix_small<uint64_t, 1>
-                            : k_radix_small<uint64_t, RSS_MAX64 / RSS_THREADS>;
+static RadixSmallFn radix_small_fn(int n) {
+    return n <= RSS_THREADS ? k_radix_small<1>
+           : n <= 4 * RSS_THREADS ? k_radix_small<4>
+           : n <= 8 * RSS_THREADS ? k_radix_small<8>
+                                  : k_radix_small<RSS_MAX / RSS_THREADS>;
 }
 
 // The dynamic shared-memory limit of k_radix_small, raised once per device.
@@ -452,12 +463,11 @@ static bool radix_small_ready() {
     }
     if (ok[dev] == 0) {
         signed char r = 1;
-        for (int passes : {4, 8})
-            for (int n : {RSS_THREADS, 4 * RSS_THREADS, passes == 4 ? RSS_MAX : RSS_MAX64})
-                if (cudaFuncSetAttribute(radix_small_fn(n, passes),
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)radix_small_smem(RSS_MAX, 4)) != cudaSuccess)
-                    r = -1;
+        for (int n : {RSS_THREADS, 4 * RSS_THREADS, 8 * RSS_THREADS, RSS_MAX})
+            if (cudaFuncSetAttribute(radix_small_fn(n),
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)radix_small_smem(RSS_MAX)) != cudaSuccess)
+                r = -1;
         if (r < 0) cudaGetLastError();
         ok[dev] = r;
     }
@@ -471,10 +481,9 @@ size_t radix_counts_elems(size_t n) {
 void radix_sort(cudaStream_t s, int n, int bits, uint64_t *key,
                 uint32_t *val, SortScratch &sc, int *launches) {
     if (n <= 1 || bits <= 0) return;
-    if (radix_small_takes(n, bits) && radix_small_ready()) {
-        const int passes = (bits + 7) / 8;
-        radix_small_fn(n, passes)<<<1, RSS_THREADS, radix_small_smem(n, passes), s>>>(
-            n, passes, key, val);
+    if (n <= RSS_MAX && radix_small_ready()) {
+        radix_small_fn(n)<<<1, RSS_THREADS, radix_small_smem(n), s>>>(n, (bits + 7) / 8, key,
+                                                                     val);
         *launches += 1;
         return;
     }
@@ -849,8 +858,7 @@ __global__ void __launch_bounds__(SS_THREADS)
     });
 }
 
-bool radix_small_takes(int n, int bits) { return n <= (bits <= 32 ? RSS_MAX : RSS_MAX64); }
-int radix_small_bytes(int n, int passes) { return (int)radix_small_smem(n, passes); }
+int radix_small_max() { return RSS_MAX; }
 bool radix_small_available() { return radix_small_ready(); }
 int scan_small_max() { return SS_MAX; }
 
@@ -877,17 +885,17 @@ void launch_keys_batch(cudaStream_t s, const KeysRec *args, const BatchSpan &sp)
     if (sp.total > 0) k_keys_batch<<<batch_grid(r, sp.total), 256, 0, s>>>(args, sp);
 }
 bool launch_radix_small_batch(cudaStream_t s, const RadixSmallRec *args, const BatchSpan &sp,
-                              int max_smem) {
+                              int max_n) {
     static const bool ok = cudaFuncSetAttribute(k_radix_small_batch,
                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)radix_small_smem(RSS_MAX, 4)) == cudaSuccess;
-    if (!ok || max_smem > (int)radix_small_smem(RSS_MAX, 4)) {
+                                                (int)radix_small_smem(RSS_MAX)) == cudaSuccess;
+    if (!ok || max_n > RSS_MAX) {
         cudaGetLastError();
         return false;
     }
     if (sp.total > 0)
-        k_radix_small_batch<<<std::min(sp.total, gpu_sms()), RSS_THREADS, (size_t)max_smem, s>>>(
-            args, sp);
+        k_radix_small_batch<<<std::min(sp.total, gpu_sms()), RSS_THREADS, radix_small_smem(max_n),
+                              s>>>(args, sp);
     return true;
 }
 void launch_scan_small_batch(cudaStream_t s, const ScanSmallRec *args, const BatchSpan &sp) {

@@ -272,15 +272,14 @@ struct ScanSmallRec {
     uint32_t *total_dev;
     int write_total_at_n;
 };
-bool radix_small_takes(int n, int bits);      // whether the single-block sort does
-int radix_small_bytes(int n, int passes);     // its dynamic shared memory
+int radix_small_max();           // largest set the single-block sort takes
 bool radix_small_available();    // its shared-memory limit could be raised
 int scan_small_max();            // largest set the single-block scan takes
 void launch_rebuild_reset_batch(cudaStream_t s, const RebuildReset *args, const BatchSpan &sp);
 void launch_keys_batch(cudaStream_t s, const KeysRec *args, const BatchSpan &sp);
 // false (nothing launched) if the shared-memory limit cannot be raised
 bool launch_radix_small_batch(cudaStream_t s, const RadixSmallRec *args, const BatchSpan &sp,
-                              int max_smem);
+                              int max_n);
 void launch_scan_small_batch(cudaStream_t s, const ScanSmallRec *args, const BatchSpan &sp);
 // cmin[start of each cell] = min of v over the cell (sorted set).
 void launch_cell_min(cudaStream_t s, int n, const uint64_t *skey,
