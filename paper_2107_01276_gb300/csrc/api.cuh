@@ -82,7 +82,19 @@ using sph::api::NFAM;
 using namespace sph;
 using namespace sph::api;
 
-struct sph_ctx {
+// What the launches of a step leave behind on the host: where the state lies
+// and what the lists are.  A replay of the captured launches sets it whole.
+struct StepHost {
+    double *f[NF] = {};      // FP64 state, current (sorted) order
+    double *falt[NF] = {};   // gather targets, swapped with f
+    int64_t *id = nullptr, *id_alt = nullptr;
+    uint32_t tmask = 0;             // slots of the cell table - 1
+    float skin = 1.0f;              // skin factor of the current lists (1: exact)
+    bool rows = false;              // the current lists have rows
+    bool wall_lists_valid = false;  // the last build made wall lists
+};
+
+struct sph_ctx : StepHost {
     sph_params prm;
     cudaStream_t s = nullptr;
     std::string err;
@@ -92,10 +104,6 @@ struct sph_ctx {
     double c0 = 0.0;
     int lmax = 0, mbits = 1, lbits = 0;
     Level lev[MAX_LEVELS];
-
-    double *f[NF] = {};      // FP64 state, current (sorted) order
-    double *falt[NF] = {};   // gather targets, swapped with f
-    int64_t *id = nullptr, *id_alt = nullptr;
 
     // pair-pass outputs and mirrors, sized for doubles (floats use half)
     void *nbA = nullptr, *nbB = nullptr;   // pass-B records (double4 sized)
@@ -112,7 +120,7 @@ struct sph_ctx {
     uint64_t *tkey = nullptr;
     uint32_t *tstart = nullptr, *tend = nullptr;
     float *tmaxh = nullptr;     // per slot: the cell's largest h
-    uint32_t tcap = 0, tmask = 0;
+    uint32_t tcap = 0;
     int *bbox = nullptr;
     uint32_t *level_mask = nullptr;
     // neighbour lists and packed per-particle data
@@ -124,7 +132,6 @@ struct sph_ctx {
     uint32_t *longq = nullptr, *d_nlong = nullptr;
     uint32_t *stage = nullptr, *lqueue = nullptr, *d_nlq = nullptr;
     uint32_t *rlen = nullptr;       // row lengths (ListArgs::rlen)
-    bool rows = false;              // the current lists have rows
     uint32_t *lqref = nullptr;      // queued particles' chunk references
     uint32_t stage_w = 64;          // staging row width (entries)
     uint32_t stage_want = 0;        // width to switch to at the next build
@@ -144,7 +151,6 @@ struct sph_ctx {
     uint32_t *wlongq = nullptr, *d_wnlong = nullptr;
     uint32_t wcap = 0;
     int wall_mode = 0;              // 0: by wall count, 1: cell walk, 2: lists
-    bool wall_lists_valid = false;  // the last build made them
     double *d_force = nullptr;   // sph_forces: 8 n_wall + 4 doubles
     int force_cap = 0;           // walls d_force holds
     double *d_mass = nullptr, *d_mass_part = nullptr;  // [2], [256]
@@ -176,7 +182,6 @@ struct sph_ctx {
     // list sizing: entry total and particle count of the last build that
     // read its total back
     uint32_t last_total[3] = {};     // per ListForm
-    float skin = 1.0f;          // skin factor of the current lists (1: exact)
     int *d_skin_err = nullptr;  // set when particles outran the skin
     int last_total_n[3] = {};
     // with rows: entries that were in them at the last such read-back
@@ -203,10 +208,7 @@ struct sph_ctx {
     struct StepGraph {
         cudaGraphExec_t exec = nullptr;
         std::vector<uintptr_t> key;              // what the launches depend on
-        double *f_after[NF], *falt_after[NF];    // buffers after the step
-        int64_t *id_after = nullptr, *id_alt_after = nullptr;
-        uint32_t tmask = 0;
-        float skin = 1.0f;
+        StepHost after;                          // the host side after the step
         int launches = 0;
     } graphs[2];
     Timer tm;

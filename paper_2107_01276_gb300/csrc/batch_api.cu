@@ -34,10 +34,7 @@ struct sph_batch {
     std::vector<uintptr_t> comp;   // contexts and configurations of the last call
     int same_comp = 0;
     struct Inst {
-        double *f_after[NF], *falt_after[NF];
-        int64_t *id_after = nullptr, *id_alt_after = nullptr;
-        uint32_t tmask = 0;
-        float skin = 1.0f;
+        StepHost after;
         int launches = 0;
     };
     struct Graph {
@@ -712,10 +709,7 @@ static bool batch_graph_step(sph_batch *b, const std::vector<sph_ctx *> &all,
             return false;
         }
         struct Saved {
-            double *f[NF], *falt[NF];
-            int64_t *id, *id_alt;
-            uint32_t tmask;
-            float skin;
+            StepHost host;
             long long steps;
             bool gv, rv;
             int launches;
@@ -723,12 +717,7 @@ static bool batch_graph_step(sph_batch *b, const std::vector<sph_ctx *> &all,
         std::vector<Saved> sv(k);
         for (size_t q = 0; q < k; ++q) {
             sph_ctx *c = all[q];
-            memcpy(sv[q].f, c->f, sizeof(c->f));
-            memcpy(sv[q].falt, c->falt, sizeof(c->falt));
-            sv[q].id = c->id;
-            sv[q].id_alt = c->id_alt;
-            sv[q].tmask = c->tmask;
-            sv[q].skin = c->skin;
+            sv[q].host = *c;
             sv[q].steps = c->steps;
             sv[q].gv = c->grid_valid;
             sv[q].rv = c->rhs_valid;
@@ -756,12 +745,7 @@ static bool batch_graph_step(sph_batch *b, const std::vector<sph_ctx *> &all,
             if (ex) cudaGraphExecDestroy(ex);
             for (size_t q = 0; q < k; ++q) {
                 sph_ctx *c = all[q];
-                memcpy(c->f, sv[q].f, sizeof(c->f));
-                memcpy(c->falt, sv[q].falt, sizeof(c->falt));
-                c->id = sv[q].id;
-                c->id_alt = sv[q].id_alt;
-                c->tmask = sv[q].tmask;
-                c->skin = sv[q].skin;
+                static_cast<StepHost &>(*c) = sv[q].host;
                 c->steps = sv[q].steps;
                 c->grid_valid = sv[q].gv;
                 c->rhs_valid = sv[q].rv;
@@ -778,12 +762,7 @@ static bool batch_graph_step(sph_batch *b, const std::vector<sph_ctx *> &all,
         for (size_t q = 0; q < k; ++q) {
             sph_ctx *c = all[q];
             sph_batch::Inst &in = slot->inst[q];
-            memcpy(in.f_after, c->f, sizeof(c->f));
-            memcpy(in.falt_after, c->falt, sizeof(c->falt));
-            in.id_after = c->id;
-            in.id_alt_after = c->id_alt;
-            in.tmask = c->tmask;
-            in.skin = c->skin;
+            in.after = *c;
             in.launches = c->launches - sv[q].launches;
         }
         slot->launches = b->launches - bl0;
@@ -792,12 +771,7 @@ static bool batch_graph_step(sph_batch *b, const std::vector<sph_ctx *> &all,
         for (size_t q = 0; q < k; ++q) {
             sph_ctx *c = all[q];
             const sph_batch::Inst &in = g->inst[q];
-            memcpy(c->f, in.f_after, sizeof(c->f));
-            memcpy(c->falt, in.falt_after, sizeof(c->falt));
-            c->id = in.id_after;
-            c->id_alt = in.id_alt_after;
-            c->tmask = in.tmask;
-            c->skin = in.skin;
+            static_cast<StepHost &>(*c) = in.after;
             c->launches += in.launches;
             c->grid_valid = false;
             c->rhs_valid = true;

@@ -77,13 +77,7 @@ bool graph_step(sph_ctx *c, sph_status *st) {
         drop_graph(*slot);
         // capture one step; the host side runs as usual, the kernels only
         // run when the graph is launched below
-        double *f0[NF], *fa0[NF];
-        memcpy(f0, c->f, sizeof(f0));
-        memcpy(fa0, c->falt, sizeof(fa0));
-        int64_t *id0 = c->id, *ida0 = c->id_alt;
-        const uint32_t tmask0 = c->tmask;
-        const float skin0 = c->skin;
-        const bool rows0 = c->rows;
+        const StepHost host0 = *c;
         const long long steps0 = c->steps;
         const bool gv0 = c->grid_valid, rv0 = c->rhs_valid;
         const int l0 = c->launches;
@@ -103,13 +97,7 @@ bool graph_step(sph_ctx *c, sph_status *st) {
             // undo the host side and run the step launch by launch
             cudaGetLastError();
             if (ex) cudaGraphExecDestroy(ex);
-            memcpy(c->f, f0, sizeof(f0));
-            memcpy(c->falt, fa0, sizeof(fa0));
-            c->id = id0;
-            c->id_alt = ida0;
-            c->tmask = tmask0;
-            c->skin = skin0;
-            c->rows = rows0;
+            static_cast<StepHost &>(*c) = host0;
             c->steps = steps0;
             c->grid_valid = gv0;
             c->rhs_valid = rv0;
@@ -120,21 +108,11 @@ bool graph_step(sph_ctx *c, sph_status *st) {
         }
         slot->exec = ex;
         slot->key = key;
-        memcpy(slot->f_after, c->f, sizeof(c->f));
-        memcpy(slot->falt_after, c->falt, sizeof(c->falt));
-        slot->id_after = c->id;
-        slot->id_alt_after = c->id_alt;
-        slot->tmask = c->tmask;
-        slot->skin = c->skin;
+        slot->after = *c;
         slot->launches = c->launches - l0;
         g = slot;
     } else {
-        memcpy(c->f, g->f_after, sizeof(c->f));
-        memcpy(c->falt, g->falt_after, sizeof(c->falt));
-        c->id = g->id_after;
-        c->id_alt = g->id_alt_after;
-        c->tmask = g->tmask;
-        c->skin = g->skin;
+        static_cast<StepHost &>(*c) = g->after;
         c->launches += g->launches;
         c->grid_valid = false;
         c->rhs_valid = true;
