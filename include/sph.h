@@ -452,8 +452,8 @@ typedef struct {
                             so steps run launch by launch.  1: always launch
                             by launch */
     /* filled by sph_autotune: mean device ms per launch of each candidate
-     * (neighbour build + both passes for cell_scale 1, 1.25, 1.5; the walk
-     * for walk 1, 2, 4; pass A / pass B for teams 1, 4, 16, 32) */
+     * (neighbour build + both passes for cell_scale 1, 1.25, 1.5 and for
+     * walk 1, 2, 4; pass A / pass B for teams 1, 4, 16, 32) */
     double ms_cell[3], ms_walk[3], ms_team_a[4], ms_team_b[4];
     double ms_walls[2];  /* build + both passes with walls 1, 2 (walls
                             loaded only) */
@@ -461,10 +461,10 @@ typedef struct {
 
 /* Autotuner (the paper has no counterpart; a launch-configuration search
  * for this GPU): on the loaded fluid set at its current state, times
- * neighbour builds and right-hand sides for each level-0 cell size
- * (x1, x1.25, x1.5), then each list-build kernel, then each team size of
- * pass A and pass B, then (with walls) the two ways the fluid sees the
- * walls (CUDA events, a few repetitions after a warm-up), and
+ * neighbour builds, as sph_step makes them, and both passes for each
+ * level-0 cell size (x1, x1.25, x1.5), then for each list-build kernel, then
+ * each team size of pass A and pass B, then (with walls) the two ways the
+ * fluid sees the walls (CUDA events, a few repetitions after a warm-up), and
  * keeps the fastest of each for this context; out (may be NULL) receives
  * the choices and the times.  It ends with a right-hand side as sph_rhs
  * does (the state re-sorted, its density the summation density, the rates

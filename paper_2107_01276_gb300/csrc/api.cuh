@@ -238,6 +238,7 @@ sph_status rebuild(sph_ctx *c, bool mid_step, bool exact = true,
 // 10 %.
 enum ListForm { LIST_EXACT, LIST_SKIN, LIST_ROWS };
 ListForm step_form(sph_ctx *c);          // of a step's first build
+float step_skin(const sph_ctx *c);       // of its lists
 // Entries of the last build of a form that read its size back.  With rows a
 // list holds the reverse entries and the own entries of particles whose rows
 // overflow: none of most sets, all of a denser one loaded after it, so a

@@ -506,7 +506,7 @@ static sph_status batch_body(sph_batch *b, const std::vector<sph_ctx *> &all,
     std::vector<sph_ctx *> rest;
     std::vector<SmallBuild> sb;
     for (sph_ctx *c : all) {
-        const float skin = is_mixed(c) ? 1.1f : 1.0f;
+        const float skin = step_skin(c);
         if (small_build_ok(c, skin)) {
             sb.emplace_back();
             plan_small_build(c, false, skin, true, sb.back());
@@ -530,7 +530,7 @@ static sph_status batch_body(sph_batch *b, const std::vector<sph_ctx *> &all,
         for (int q = a; q < e; ++q) {
             sph_ctx *c = rest[q];
             compute_dt(c, c->d_t, 1);
-            if ((bst[q] = rebuild(c, false, true, is_mixed(c) ? 1.1f : 1.0f, true, true)) != SPH_OK) return;
+            if ((bst[q] = rebuild(c, false, true, step_skin(c), true, true)) != SPH_OK) return;
         }
     };
     if (capturing)

@@ -241,6 +241,8 @@ bool want_wall_lists(const sph_ctx *c) {
     return c->wall.n >= 2048;
 }
 
+float step_skin(const sph_ctx *c) { return is_mixed(c) ? 1.1f : 1.0f; }
+
 ListForm step_form(sph_ctx *c) {
     if (!is_mixed(c)) return LIST_EXACT;
     return list_rows_for(list_args(c)) ? LIST_ROWS : LIST_SKIN;
@@ -1045,14 +1047,14 @@ static void forces_launch(sph_ctx *c) {
 // lists would cost more FP64 pair work than the build they save).  exact:
 // the first build may read the list size back.
 sph_status pec_step(sph_ctx *c, bool exact) {
-    const float step_skin = is_mixed(c) ? 1.1f : 1.0f;
+    const float skin = step_skin(c);
     compute_dt(c, c->d_t, 1);
-    sph_status st = rebuild(c, false, exact, step_skin, true, true);
+    sph_status st = rebuild(c, false, exact, skin, true, true);
     if (st != SPH_OK) return st;
     run_passes(c);
     run_pec(c, 0.5);   // (mixed: and the records of the predicted state)
     swap_stage(c);
-    if (!(step_skin > 1.0f)) {
+    if (!(skin > 1.0f)) {
         st = rebuild(c, true, false);
         if (st != SPH_OK) return st;
     }

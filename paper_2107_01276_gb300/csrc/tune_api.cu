@@ -57,8 +57,9 @@ sph_status sph_autotune(sph_ctx *c, sph_tune *out) {
     cur.no_graphs = c->use_graphs ? 0 : 1;
     cur.walls = c->wall_mode;
     sph_tune res = cur;
-    // mean ms per launch of families 0 (pass B), 1 (pass A), 2 (build), 5
-    // (walk) over `reps` builds + right-hand sides, after one untimed
+    // mean ms per launch of families 0 (pass B), 1 (pass A), 2 (build) over
+    // `reps` evaluations as a step's first one (its lists, with their skin
+    // and rows), after one untimed
     sph_status st = SPH_OK;
     auto measure = [&](int reps, double fam_ms[NFAM]) -> sph_status {
         for (int r = 0; r <= reps; ++r) {
@@ -69,7 +70,7 @@ sph_status sph_autotune(sph_ctx *c, sph_tune *out) {
             }
             compute_dt(c, nullptr, 0);
             c->grid_valid = false;
-            sph_status s2 = rebuild(c, false);
+            sph_status s2 = rebuild(c, false, true, step_skin(c), true, true);
             if (s2 != SPH_OK) return s2;
             run_passes(c);
         }
@@ -100,13 +101,14 @@ sph_status sph_autotune(sph_ctx *c, sph_tune *out) {
     // 2. list build
     if (st == SPH_OK) {
         best = -1;
-        // the team walk, the 4-lane cell tiles, the merged cell tiles
+        // the team walk, the 4-lane cell tiles, the merged cell tiles; with
+        // the passes, since the walk also decides how they read its lists
         const int walks[3] = {1, 2, 4};
         for (int q = 0; q < 3 && st == SPH_OK; ++q) {
             c->walk_choice = walks[q];
             if ((st = measure(reps, fm)) != SPH_OK) break;
-            res.ms_walk[q] = fm[5];
-            if (best < 0 || fm[5] < res.ms_walk[best]) best = q;
+            res.ms_walk[q] = fm[2] + fm[1] + fm[0];
+            if (best < 0 || res.ms_walk[q] < res.ms_walk[best]) best = q;
         }
         cur.walk = walks[best < 0 ? 0 : best];
         c->walk_choice = cur.walk;
