@@ -106,7 +106,8 @@ struct sph_ctx : StepHost {
     Level lev[MAX_LEVELS];
 
     // pair-pass outputs and mirrors, sized for doubles (floats use half)
-    void *nbA = nullptr, *nbB = nullptr;   // pass-B records (double4 sized)
+    // pass-B records (double4 sized; nbB of FP64 contexts only)
+    void *nbA = nullptr, *nbB = nullptr;
     void *rhoR = nullptr, *beta = nullptr, *pavg = nullptr, *drx = nullptr,
          *dry = nullptr, *V = nullptr, *rb2 = nullptr, *dpdt = nullptr,
          *dudt = nullptr, *dvdt = nullptr;

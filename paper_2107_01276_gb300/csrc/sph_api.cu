@@ -879,7 +879,9 @@ sph_status new_ctx(const sph_params *p, cudaStream_t stream, bool has_ds,
                      (double **)&c->rb2, (double **)&c->dpdt, (double **)&c->dudt,
                      (double **)&c->dvdt};
     for (auto pp : rs) ok = ok && dalloc(pp, N, c->s);
-    ok = ok && dalloc((double4_32a **)&c->nbA, N, c->s) && dalloc((double4_32a **)&c->nbB, N, c->s);
+    // (FP32: both records of a particle lie in nbA)
+    ok = ok && dalloc((double4_32a **)&c->nbA, N, c->s) &&
+         (is_mixed(c) || dalloc((double4_32a **)&c->nbB, N, c->s));
     ok = ok && dalloc(&c->mf, N, c->s) && dalloc(&c->pf, N, c->s) && dalloc(&c->uf, N, c->s) &&
          dalloc(&c->vf, N, c->s) && dalloc(&c->nnb, N, c->s);
     ok = ok && dalloc(&c->skey, N, c->s) && dalloc(&c->perm, N, c->s) &&
