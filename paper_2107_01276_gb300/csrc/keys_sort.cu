@@ -29,8 +29,8 @@ __device__ __forceinline__ int cell_coord(double x, double lo, double w,
                                           int ncell) {
     double q = floor(__ddiv_rn(__dsub_rn(x, lo), w));
     int c;
-    if (q < 0.0)
-        c = 0;
+    if (!(q >= 0.0))   // a NaN too, which converts to the least integer and
+        c = 0;         // would stretch the level's box to it
     else if (q > (double)(ncell - 1))
         c = ncell - 1;
     else

@@ -1,5 +1,6 @@
 """Neighbour-list storage: builds without a size read-back that run out of
-it, and sets loaded into a context whose sizes come from another set."""
+it, sets loaded into a context whose sizes come from another set, and the
+cells of particles whose positions are lost."""
 import numpy as np
 import pytest
 
@@ -113,3 +114,27 @@ def test_reloaded_context_takes_a_set_whose_rows_overflow(second):
         for f in ("u", "v", "p"):
             change = np.abs(b[f] - pt[f]).max()
             assert np.abs(a[f] - b[f]).max() <= k * MIXED_TOL * change, f
+
+
+@pytest.mark.parametrize("walk", [1, 2, 3, 4])
+@pytest.mark.parametrize("precision", [sph.SPH_FP64, sph.SPH_MIXED])
+def test_nan_positions_leave_the_cells_of_the_others_alone(precision, walk):
+    """A NaN pressure makes the positions around it NaN within a step.  In
+    the next build they count for cell 0: the walks over a level of two by
+    two cells, all of them in reach, still find the other particles, which
+    stay finite."""
+    d = wl.taylor_green(nx=50, jitter=0.1, seed=4)
+    pt = dict(d["particles"], p=d["particles"]["p"].copy())
+    pt["p"][1275] = np.nan
+    s = _sim(dict(d, particles=pt), precision, cell_c0=0.4)
+    s.set_tuning(walk=walk)
+    for _ in range(2):
+        with pytest.raises(sph.SphError) as e:
+            s.step(1)
+        assert e.value.status == sph.SPH_ENONFINITE
+    got = by_id(s, STATE)
+    s.close()
+    bad = ~np.isfinite(got["x"])
+    assert 1 < bad.sum() < 400
+    for f in STATE:
+        assert np.isfinite(got[f][pt["y"] < 0.2]).all(), f
