@@ -450,6 +450,17 @@ struct Anchor {
     int periodic[2];
 };
 
+// One axis of the lattice: n < 2^16 cells of side A.
+inline void set_anchor_axis(Anchor &an, int ax, double A, int n, bool periodic) {
+    an.A[ax] = (float)A;
+    an.iA[ax] = (float)(1.0 / A);
+    an.n[ax] = n;
+    an.periodic[ax] = periodic ? 1 : 0;
+    an.nf[ax] = periodic ? (float)n : 0.0f;
+    // below 1 / n (a tie k = n / 2 then stays unwrapped)
+    an.invn[ax] = periodic ? nextafterf((float)(1.0 / (double)n), 0.0f) : 0.0f;
+}
+
 // The anchor indices of a record as floats 2^23 + g (one byte permute each;
 // their differences are exact).
 __device__ __forceinline__ float anchor_gx(unsigned g) {

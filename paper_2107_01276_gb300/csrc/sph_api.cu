@@ -977,13 +977,7 @@ sph_status setup_fluid_grid(sph_ctx *c, long long n, double hmin,
             na = std::max(1ll, (long long)ceil(L / Ad[a]));
             if (na > 65535) na = 65535;
         }
-        an.A[a] = (float)Ad[a];
-        an.iA[a] = (float)(1.0 / Ad[a]);
-        an.n[a] = (int)na;
-        an.periodic[a] = c->dom.periodic[a];
-        an.nf[a] = an.periodic[a] ? (float)na : 0.0f;
-        // below 1 / na (a tie k = na / 2 then stays unwrapped)
-        an.invn[a] = an.periodic[a] ? nextafterf((float)(1.0 / (double)na), 0.0f) : 0.0f;
+        set_anchor_axis(an, a, Ad[a], (int)na, c->dom.periodic[a] != 0);
     }
     c->an = an;
     c->anchor_A[0] = Ad[0];
