@@ -56,12 +56,17 @@ __device__ __forceinline__ float frsqrt(float x) { return rsqrtf(x); }
 // root cost it tens of instructions a pair, these three and five.
 //
 // Sets with walls keep the correctly rounded sequence, operation for
-// operation.  They are the adaptive flows, and adaptation amplifies a last
-// bit: a split parent's children sit on a hexagon, whose equal distances
-// the merge search orders by their rounding, so after one bit the flow
-// splits and merges other particles.  Their sums are a small part of an
-// adaptive step (pass A and B 7 % of one of the 1:250 cylinder, 91k
-// particles), and their runs keep their particle history.
+// operation.  The rule looks at the walls alone; its reason is adaptation,
+// which amplifies a last bit: a split parent's children sit on a hexagon,
+// whose equal distances the merge search orders by their rounding, so after
+// one bit the flow splits and merges other particles.  The flows past bodies
+// adapt and have walls, their pair sums are a small part of an adaptive step
+// (pass A and B 7 % of one of the 1:250 cylinder, 91k particles), and they
+// keep their particle history.  The rule is not the reason on either side of
+// it: a flow that adapts without walls (a vortex with a refined region, the
+// background construction) takes these sums, and splits and merges by their
+// rounding, not by the divisions'; a walled flow that never adapts (a
+// channel) takes the slower sums.
 template <typename R, bool LEAN>
 constexpr bool lean64 = LEAN && sizeof(R) == 8;
 
@@ -132,9 +137,9 @@ __device__ __forceinline__ bool is_normal(double x) {
 // Mixed pair sums of sets without walls (LEAN): two values share an
 // instruction where the formulas come in pairs: the axes of a separation, u
 // and v, the kernels of h_i and h_j.  Each half rounds like the scalar
-// operation.  At 1M particles of the 1:250 strip pass B issues 215M warp
-// instructions and is bound by issue (72 % busy) and by the L1 data pipe of
-// its record gathers (85 %).
+// operation.  At 1M particles of the 1:250 strip pass B issues 178M warp
+// instructions and is bound by the L1 data pipe of its record gathers (83 %
+// of the peak; issue 59 %), pass A 206M and by issue (69 %; data pipe 46 %).
 struct F2 {
     unsigned long long v;
 };

@@ -23,7 +23,8 @@ namespace sph {
 // for (measured at 4.2M on the graded strip: pass A at seven and eight
 // blocks 0.92 and 1.05 ms, pass B at five, six, seven 0.92, 0.93, 1.52 ms;
 // with too few registers the loads of an iteration are no longer in flight
-// together)
+// together).  At the bound of five pass B takes 80 registers, so six are
+// resident.
 constexpr int PASS_A_BLOCKS = 7;
 constexpr int PASS_B_BLOCKS = 5;
 // Team forms (T > 1: small and walled sets) and the batched forms keep six
