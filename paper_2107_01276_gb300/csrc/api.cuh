@@ -187,10 +187,10 @@ struct sph_ctx : StepHost {
     int last_total_n[3] = {};
     // with rows: entries that were in them at the last such read-back
     unsigned long long last_rows = 0, *d_rows = nullptr;
-    // fluid sets loaded so far; the last one's count and least and largest h
+    // fluid sets loaded so far; least and largest h of the first one of the
+    // kind the sizes belong to
     int loads = 0;
-    long long load_n = -1;
-    double load_h[2] = {};
+    double sized_h[2] = {};
     long long steps = 0;
     int launches = 0;
     bool timing = false;

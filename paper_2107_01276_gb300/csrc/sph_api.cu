@@ -1206,13 +1206,18 @@ sph_status sph_load_particles(sph_ctx *c, sph_kind kind, long long n,
     std::swap(c->id, c->id_alt);
     c->n = (int)n;
     c->next_id = n > 0 && src->id ? chk.idmax + 1 : n;
-    // another kind of set: the sizes of the old one's lists say nothing
-    if (n != c->load_n || hmin != c->load_h[0] || hmax != c->load_h[1])
+    // another kind of set: the sizes of the old one's lists say nothing.  (The
+    // same with h changed a little keeps them, or a state reloaded every step
+    // would build with a read-back each time and outside the batched build:
+    // h within 10 % and list_sized's 10 % of n make at most 1.8 times the
+    // entries of the last read-back, and the list has room for twice those.)
+    if (!(hmin >= 0.9 * c->sized_h[0] && hmin <= 1.1 * c->sized_h[0] &&
+          hmax >= 0.9 * c->sized_h[1] && hmax <= 1.1 * c->sized_h[1])) {
         memset(c->last_total, 0, sizeof(c->last_total));
+        c->sized_h[0] = hmin;
+        c->sized_h[1] = hmax;
+    }
     c->loads += 1;
-    c->load_n = n;
-    c->load_h[0] = hmin;
-    c->load_h[1] = hmax;
     // a new state: a non-finite rate, skin overrun or list overflow of the
     // old one no longer applies
     cudaMemsetAsync(c->d_nonfinite, 0, sizeof(int), c->s);
