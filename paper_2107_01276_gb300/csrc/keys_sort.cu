@@ -291,11 +291,13 @@ __global__ void __launch_bounds__(RS_THREADS)
 // with __match_any_sync against per-(warp, digit) counts, scans the counts
 // digit-major (a warp takes 8 digits, a lane a warp's count), scatters keys
 // and positions into shared memory and reloads them in the new order, so
-// the sort is stable exactly like the tiled form.  A key travels as 32 bits:
-// its low word through the first four passes; a wider key's high word is
-// then fetched from its place in the input, and the whole key at the end
-// (64-bit keys in registers left room for half the items, and wide sets of
-// 8193 to 16384 particles to the tiled sort's fifteen launches or more).
+// the sort is stable exactly like the tiled form.  A key travels whole where
+// that is 32 bits, or 64 and n <= RSS_MAX / 2.  TWO: as one 32-bit word for
+// any width up to RSS_MAX, the low one through the first four passes, then
+// the high one, fetched from its place in the input, and the whole key at the
+// end (64-bit keys leave room for half the items; wide sets of 8193 to 16384
+// particles would go to the tiled sort's fifteen launches or more: 12000, 100
+// -> 57 us a call.  Up to a thousand, whole keys save the two fetches, 1 us).
 // Bound by the latency of its chain of passes: 5 us at 2.5k particles and 3
 // digits, 9.5 us at 16k (the former form, with two rankings a pass and
 // passes through global memory, took 10 and 29).
@@ -303,20 +305,22 @@ constexpr int RSS_THREADS = 1024;
 constexpr int RSS_WARPS = RSS_THREADS / 32;
 constexpr int RSS_MAX = 16384;
 
-static size_t radix_small_smem(int n) { return (size_t)n * 6; }
+// dynamic shared memory: key words and 16-bit positions
+static size_t radix_small_smem(int n, bool whole64) { return (size_t)n * (whole64 ? 10 : 6); }
+static bool radix_small_whole64(int n, int passes) { return passes > 4 && n <= RSS_MAX / 2; }
 
-template <int IT>
+template <typename K, int IT, bool TWO>
 __device__ __forceinline__ void radix_small_body(int n, int passes, uint64_t *ka,
                                                  uint32_t *va, uint32_t (*cnt)[257],
                                                  uint32_t *dtot) {
     extern __shared__ uint64_t rss_buf[];          // n key words, then n positions
-    uint32_t *sk = (uint32_t *)rss_buf;
+    K *sk = (K *)rss_buf;
     uint16_t *si = (uint16_t *)(sk + n);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const int rows = (n + RSS_THREADS - 1) / RSS_THREADS;   // items a lane, <= IT
     const int wb = w * rows * 32 + lane;
-    uint32_t key[IT];
+    K key[IT];
     uint32_t ir[IT];                               // position | rank << 16
 #pragma unroll
     for (int s = 0; s < IT; ++s) {
@@ -324,16 +328,16 @@ __device__ __forceinline__ void radix_small_body(int n, int passes, uint64_t *ka
         key[s] = 0;
         ir[s] = 0;
         if (s < rows && e < n) {
-            key[s] = (uint32_t)ka[e];
+            key[s] = (K)ka[e];
             ir[s] = (uint32_t)e;
         }
     }
     for (int p = 0; p < passes; ++p) {
-        const int shift = 8 * (p & 3);
-        if (p == 4) {
+        const int shift = 8 * (TWO ? p & 3 : p);
+        if (TWO && p == 4) {
 #pragma unroll
             for (int s = 0; s < IT; ++s)
-                if (s < rows && wb + s * 32 < n) key[s] = (uint32_t)(ka[ir[s]] >> 32);
+                if (s < rows && wb + s * 32 < n) key[s] = (K)(ka[ir[s]] >> 32);
         }
         for (int t = threadIdx.x; t < RSS_WARPS * 257; t += RSS_THREADS) (&cnt[0][0])[t] = 0;
         __syncthreads();
@@ -406,7 +410,7 @@ __device__ __forceinline__ void radix_small_body(int n, int passes, uint64_t *ka
         }
     }
     // the keys and values of the final order, all read before any is replaced
-    if (passes > 4) {   // (the low words wait in shared memory)
+    if (TWO && passes > 4) {   // (the low words wait in shared memory)
 #pragma unroll
         for (int s = 0; s < IT; ++s)
             if (s < rows && wb + s * 32 < n) sk[wb + s * 32] = (uint32_t)ka[ir[s]];
@@ -432,25 +436,32 @@ __device__ __forceinline__ void radix_small_body(int n, int passes, uint64_t *ka
 __device__ __forceinline__ void radix_small_at(int n, int passes, uint64_t *ka, uint32_t *va) {
     __shared__ uint32_t cnt[RSS_WARPS][257];       // padded: a lane a row is conflict-free
     __shared__ uint32_t dtot[256];
-    radix_small_body<RSS_MAX / RSS_THREADS>(n, passes, ka, va, cnt, dtot);
+    radix_small_body<uint32_t, RSS_MAX / RSS_THREADS, true>(n, passes, ka, va, cnt, dtot);
 }
 
 // Alone, the sort is compiled for the items a lane really has: the unrolled
 // 16 of the largest sets are many times the instructions that a set of a
 // thousand needs, and their fetching was most of its time.
-template <int IT>
+template <typename K, int IT, bool TWO>
 __global__ void __launch_bounds__(RSS_THREADS)
     k_radix_small(int n, int passes, uint64_t *ka, uint32_t *va) {
     __shared__ uint32_t cnt[RSS_WARPS][257];
     __shared__ uint32_t dtot[256];
-    radix_small_body<IT>(n, passes, ka, va, cnt, dtot);
+    radix_small_body<K, IT, TWO>(n, passes, ka, va, cnt, dtot);
 }
 using RadixSmallFn = void (*)(int, int, uint64_t *, uint32_t *);
-static RadixSmallFn radix_small_fn(int n) {
-    return n <= RSS_THREADS ? k_radix_small<1>
-           : n <= 4 * RSS_THREADS ? k_radix_small<4>
-           : n <= 8 * RSS_THREADS ? k_radix_small<8>
-                                  : k_radix_small<RSS_MAX / RSS_THREADS>;
+template <typename K, bool TWO>
+static RadixSmallFn radix_small_fn_of(int n) {
+    constexpr int MOST = sizeof(K) == 8 ? 8 : RSS_MAX / RSS_THREADS;
+    return n <= RSS_THREADS ? k_radix_small<K, 1, TWO>
+           : n <= 4 * RSS_THREADS ? k_radix_small<K, 4, TWO>
+           : n <= 8 * RSS_THREADS ? k_radix_small<K, 8, TWO>
+                                  : k_radix_small<K, MOST, TWO>;
+}
+static RadixSmallFn radix_small_fn(int n, int passes) {
+    if (passes <= 4) return radix_small_fn_of<uint32_t, false>(n);
+    if (radix_small_whole64(n, passes)) return radix_small_fn_of<uint64_t, false>(n);
+    return k_radix_small<uint32_t, RSS_MAX / RSS_THREADS, true>;
 }
 
 // The dynamic shared-memory limit of k_radix_small, raised once per device.
@@ -463,11 +474,12 @@ static bool radix_small_ready() {
     }
     if (ok[dev] == 0) {
         signed char r = 1;
-        for (int n : {RSS_THREADS, 4 * RSS_THREADS, 8 * RSS_THREADS, RSS_MAX})
-            if (cudaFuncSetAttribute(radix_small_fn(n),
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)radix_small_smem(RSS_MAX)) != cudaSuccess)
-                r = -1;
+        for (int passes : {4, 8})
+            for (int n : {RSS_THREADS, 4 * RSS_THREADS, 8 * RSS_THREADS, RSS_MAX})
+                if (cudaFuncSetAttribute(radix_small_fn(n, passes),
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)radix_small_smem(RSS_MAX, false)) != cudaSuccess)
+                    r = -1;
         if (r < 0) cudaGetLastError();
         ok[dev] = r;
     }
@@ -482,8 +494,10 @@ void radix_sort(cudaStream_t s, int n, int bits, uint64_t *key,
                 uint32_t *val, SortScratch &sc, int *launches) {
     if (n <= 1 || bits <= 0) return;
     if (n <= RSS_MAX && radix_small_ready()) {
-        radix_small_fn(n)<<<1, RSS_THREADS, radix_small_smem(n), s>>>(n, (bits + 7) / 8, key,
-                                                                     val);
+        const int passes = (bits + 7) / 8;
+        radix_small_fn(n, passes)<<<1, RSS_THREADS,
+                                    radix_small_smem(n, radix_small_whole64(n, passes)), s>>>(
+            n, passes, key, val);
         *launches += 1;
         return;
     }
@@ -888,13 +902,13 @@ bool launch_radix_small_batch(cudaStream_t s, const RadixSmallRec *args, const B
                               int max_n) {
     static const bool ok = cudaFuncSetAttribute(k_radix_small_batch,
                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)radix_small_smem(RSS_MAX)) == cudaSuccess;
+                                                (int)radix_small_smem(RSS_MAX, false)) == cudaSuccess;
     if (!ok || max_n > RSS_MAX) {
         cudaGetLastError();
         return false;
     }
     if (sp.total > 0)
-        k_radix_small_batch<<<std::min(sp.total, gpu_sms()), RSS_THREADS, radix_small_smem(max_n),
+        k_radix_small_batch<<<std::min(sp.total, gpu_sms()), RSS_THREADS, radix_small_smem(max_n, false),
                               s>>>(args, sp);
     return true;
 }
